@@ -8,6 +8,8 @@
 // coarse_fused.cuh), bitwise the same as the launch sequence.
 #include "coarse_fused.cuh"
 
+#include <atomic>
+
 namespace h3d {
 namespace {
 
@@ -17,6 +19,30 @@ __global__ void __launch_bounds__(512) k_vcycle_small(SmallArgs<T> a) {
   const int item = blockIdx.x;
   if (a.active && !a.active[item]) return;
   vcycle_small_body<T, ORDER>(a, item, reinterpret_cast<T*>(smem_raw));
+}
+
+// shared memory of the deepest case, all levels from kFusedMaxN down
+constexpr size_t small_smem_max(size_t tsize) {
+  size_t n = 0;
+  for (int N = kFusedMaxN; N >= 1; N = (N - 1) / 2) n += 3 * (size_t)N * N * N;
+  return n * tsize;
+}
+
+template <typename T, int ORDER>
+cudaError_t launch_small(const SmallArgs<T>& a, int B, size_t smem, cudaStream_t st) {
+  // the shared-memory opt-in once per process (one device) and for every
+  // depth: the call waits for other streams' kernels, up to a tenth of a
+  // second when they keep the GPU full
+  static std::atomic<bool> set{false};
+  if (!set.load()) {
+    cudaError_t e = cudaFuncSetAttribute(k_vcycle_small<T, ORDER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)small_smem_max(sizeof(T)));
+    if (e != cudaSuccess) return e;
+    set.store(true);
+  }
+  k_vcycle_small<T, ORDER><<<B, 512, smem, st>>>(a);
+  count_launch();
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -46,18 +72,8 @@ cudaError_t launch_vcycle_small(int order, int nlev, const int* Ns, const Coef<T
   a.nu2 = nu2;
   a.active = active;
   const size_t smem = vcycle_small_smem(nlev, Ns, sizeof(T));
-  cudaError_t err;
-  if (order == 2) {
-    err = cudaFuncSetAttribute(k_vcycle_small<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
-    k_vcycle_small<T, 2><<<B, 512, smem, st>>>(a);
-  } else {
-    err = cudaFuncSetAttribute(k_vcycle_small<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
-    k_vcycle_small<T, 4><<<B, 512, smem, st>>>(a);
-  }
-  count_launch();
-  return cudaGetLastError();
+  if (smem > small_smem_max(sizeof(T))) return cudaErrorInvalidValue;
+  return order == 2 ? launch_small<T, 2>(a, B, smem, st) : launch_small<T, 4>(a, B, smem, st);
 }
 
 template cudaError_t launch_vcycle_small<double>(int, int, const int*, const Coef<double>* const*, int,

@@ -29,6 +29,7 @@
 // launch guarantees that all blocks are resident at once.
 
 #include <algorithm>
+#include <atomic>
 
 #include "../../include/heat3d.h"
 #include "coarse_fused.cuh"
@@ -473,20 +474,29 @@ __global__ void k_barrier_selftest(PersistCtl* ctl, int absent, int* out) {
 template <typename T, int ORDER>
 cudaError_t launch_order(const PersistArgs<T>& A, int nblk, size_t smem, cudaStream_t st) {
   auto kern = k_mg_persist<T, ORDER>;
-  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (err != cudaSuccess) return err;
-  int dev = 0, nsm = 0, per_sm = 0;
-  if ((err = cudaGetDevice(&dev)) != cudaSuccess) return err;
-  if ((err = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-    return err;
-  err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPersistThreads, smem);
-  if (err != cudaSuccess) return err;
-  if (per_sm < 1) return cudaErrorCooperativeLaunchTooLarge;
-  nblk = std::max(1, std::min(nblk, per_sm * nsm));
+  // shared-memory opt-in and resident blocks, once per process (one device)
+  // for the largest shared memory seen: host work of every small solve else
+  static std::atomic<int> slots{0};
+  static std::atomic<size_t> opted{0};
+  if (slots.load() == 0 || opted.load() < smem) {
+    const size_t want = std::max(smem, opted.load());
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)want);
+    if (err != cudaSuccess) return err;
+    int dev = 0, nsm = 0, per_sm = 0;
+    if ((err = cudaGetDevice(&dev)) != cudaSuccess) return err;
+    if ((err = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+      return err;
+    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPersistThreads, want);
+    if (err != cudaSuccess) return err;
+    if (per_sm < 1) return cudaErrorCooperativeLaunchTooLarge;
+    slots.store(per_sm * nsm);
+    opted.store(want);
+  }
+  nblk = std::max(1, std::min(nblk, slots.load()));
   PersistArgs<T> arg = A;
   void* args[] = {&arg};
-  err = cudaLaunchCooperativeKernel((const void*)kern, dim3(nblk), dim3(kPersistThreads), args,
-                                    smem, st);
+  cudaError_t err = cudaLaunchCooperativeKernel((const void*)kern, dim3(nblk), dim3(kPersistThreads),
+                                                args, smem, st);
   count_launch();
   return err;
 }

@@ -16,6 +16,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <initializer_list>
 #include <vector>
 
 #include "../../include/heat3d.h"
@@ -1322,50 +1323,96 @@ int h3d_run(heat3d_ctx* c, double* ucur, heat3d_stats* s) {
 // autotuner: launch shape per multigrid level (all shapes give identical results)
 // ---------------------------------------------------------------------------
 
-template <typename Launch>
-static float time_shape(heat3d_ctx* c, cudaEvent_t e0, cudaEvent_t e1, Launch&& launch) {
-  if (launch() != cudaSuccess) return 1e30f;  // warm-up
-  float best = 1e30f;
-  for (int rep = 0; rep < 3; ++rep) {
-    cudaEventRecord(e0, c->st);
-    cudaError_t e = launch();
-    cudaEventRecord(e1, c->st);
-    if (e != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess) return 1e30f;
-    float ms = 0.f;
-    cudaEventElapsedTime(&ms, e0, e1);
-    best = std::min(best, ms);
+// Times every candidate of one kernel: a warm-up launch and three timed ones
+// each, enqueued for a group of candidates before the first wait, so that
+// tuning costs the kernels' own time and not a host round trip per launch (a
+// context that is set up while others run, as a serving group is, would wait
+// behind their kernels at each).  Few events, kept from one kernel to the
+// next: creating hundreds makes the driver allocate, and that waits for the
+// other streams.  best[q]: the shortest time of candidate q in ms, 1e30 for
+// one that could not be launched.
+class ShapeTimer {
+ public:
+  ~ShapeTimer() {
+    for (cudaEvent_t e : ev_) cudaEventDestroy(e);
   }
-  return best;
-}
+  template <typename Launch>
+  cudaError_t run(int n, cudaStream_t st, std::vector<float>& best, Launch&& launch) {
+    best.assign(n, 1e30f);
+    while (ev_.size() < kGroup * kEvents) {
+      cudaEvent_t e;
+      cudaError_t rc = cudaEventCreate(&e);
+      if (rc != cudaSuccess) return rc;
+      ev_.push_back(e);
+    }
+    for (int q0 = 0; q0 < n; q0 += kGroup) {
+      const int m = std::min<int>(kGroup, n - q0);
+      bool ok[kGroup];
+      for (int q = 0; q < m; ++q) {
+        const cudaEvent_t* e = ev_.data() + kEvents * q;
+        ok[q] = launch(q0 + q) == cudaSuccess;  // warm-up
+        for (int r = 0; ok[q] && r < kEvents; ++r) {
+          ok[q] = cudaEventRecord(e[r], st) == cudaSuccess;
+          if (ok[q] && r + 1 < kEvents) ok[q] = launch(q0 + q) == cudaSuccess;
+        }
+      }
+      cudaError_t rc = cudaStreamSynchronize(st);
+      if (rc != cudaSuccess) return rc;
+      for (int q = 0; q < m; ++q)
+        for (int r = 0; ok[q] && r + 1 < kEvents; ++r) {
+          float ms = 0.f;
+          const cudaEvent_t* e = ev_.data() + kEvents * q;
+          if (cudaEventElapsedTime(&ms, e[r], e[r + 1]) == cudaSuccess) best[q0 + q] = std::min(best[q0 + q], ms);
+        }
+    }
+    return cudaSuccess;
+  }
+
+ private:
+  static constexpr int kGroup = 8, kEvents = 4;
+  std::vector<cudaEvent_t> ev_;
+};
 
 static bool tune_log() {
   const char* v = getenv("HEAT3D_TUNE_LOG");
   return v && v[0] == '1';
 }
 
-// vec4: the operator has the four-points-per-thread FP32 tiles (kinds 7-14,
-// and 15-26 with the z neighbours in registers, 19-26 loading planes by
-// TMA, 23-26 with a producer warp and no block barriers); the latter also
-// try a chunk of 12 planes and the chunks that fill one or two whole waves
-// of the GPU.
+// The launch shapes worth timing.  vec4: the operator has the
+// four-points-per-thread FP32 tiles (kinds 7-14, and 15-26 with the z
+// neighbours in registers, 19-26 loading planes by TMA, 23-26 with a producer
+// warp and no block barriers); the latter also try the chunks that fill one or
+// two whole waves of the GPU.  Kinds and chunks that never came within a few
+// percent of the best on a class of grids are left out of it (the deep rings
+// below 127, the one-point tiles' long chunks, kinds 11, 13, 14, 17, 21, 26):
+// a context that is set up beside busy streams pays for every launch here.
 static std::vector<Shape> shape_candidates(int N, bool vec4) {
   std::vector<Shape> v;
-  for (int zc : {1, 2, 4, 8, 16, 32, 64})
-    if (zc <= N) v.push_back(Shape{1, zc});
-  if (N >= 16) {
-    for (int kind = 2; kind <= (vec4 ? 14 : 6); ++kind)
-      for (int zc : {2, 4, 8, 16, 32, 64})
+  auto add = [&](std::initializer_list<int> kinds, std::initializer_list<int> chunks) {
+    for (int kind : kinds)
+      for (int zc : chunks)
         if (zc <= N) v.push_back(Shape{kind, zc});
-    if (vec4)  // zc -1, -2: the chunk length that fills one or two whole waves
-      for (int kind = 15; kind <= 26; ++kind)
-        for (int zc : {8, 12, 16, 32, -1, -2})
-          if (zc <= N) v.push_back(Shape{kind, zc});
+  };
+  add({1}, {1, 2, 4, 8});
+  if (N < 16) return v;
+  add({2, 4, 5}, {2, 4, 8});
+  if (!vec4) {
+    if (N >= 127) add({3, 4, 5, 6}, {16, 32, 64});
+    return v;
+  }
+  if (N < 127) {
+    add({7, 8, 9}, {4, 8});
+    add({16, 20, 24}, {8, -1});
+  } else {
+    add({7, 8, 9, 10, 12}, {4, 8, 16, 32});
+    add({15, 16, 18, 19, 20, 22, 23, 24, 25}, {8, 16, -1, -2});
   }
   return v;
 }
 
 template <typename T>
-static int autotune_T(heat3d_ctx* c, cudaEvent_t e0, cudaEvent_t e1) {
+static int autotune_T(heat3d_ctx* c, ShapeTimer& timer) {
+  std::vector<float> ms;
   for (int lev = 0; lev < c->cfg.nlevels; ++lev) {
     SdcLevel& L = c->lv[lev];
     for (int k = 0; k < L.nmg; ++k) {
@@ -1374,30 +1421,28 @@ static int autotune_T(heat3d_ctx* c, cudaEvent_t e0, cudaEvent_t e1) {
       T* b = mgbuf<T>(L, k, 0, 0);
       T* e = mgbuf<T>(L, k, 1, 0);
       T* t = mgbuf<T>(L, k, 2, 0);
-      float best = 1e30f;
-      Shape pick{1, std::min(16, g.N)};
-      for (Shape sh : shape_candidates(g.N, sizeof(T) == 4)) {
-        float ms = time_shape(c, e0, e1, [&] {
-          return launch_jacobi<T>(L.L.order, g, L.B, e, b, t, nullptr, 0, cf, nullptr, sh, c->st);
-        });
-        if (tune_log())
+      const std::vector<Shape> cand = shape_candidates(g.N, sizeof(T) == 4);
+      L.shapeT[k] = cand[0];
+      if (cand.size() < 2) continue;
+      CK(timer.run((int)cand.size(), c->st, ms, [&](int q) {
+        return launch_jacobi<T>(L.L.order, g, L.B, e, b, t, nullptr, 0, cf, nullptr, cand[q], c->st);
+      }));
+      if (tune_log())
+        for (size_t q = 0; q < cand.size(); ++q)
           fprintf(stderr, "tune jacobi T%zu order %d N %d B %d kind %d zc %d: %.4f ms\n", sizeof(T),
-                  L.L.order, g.N, L.B, sh.kind, sh.zc, ms);
-        if (ms < best) { best = ms; pick = sh; }
-      }
-      L.shapeT[k] = pick;
+                  L.L.order, g.N, L.B, cand[q].kind, cand[q].zc, ms[q]);
+      L.shapeT[k] = cand[std::min_element(ms.begin(), ms.end()) - ms.begin()];
     }
-    float best = 1e30f;
-    Shape pick{1, std::min(16, L.g.N)};
     const long long fs = L.g.fs;
-    for (Shape sh : shape_candidates(L.g.N, false)) {
-      float ms = time_shape(c, e0, e1, [&] {
+    const std::vector<Shape> cand = shape_candidates(L.g.N, false);
+    L.shape64 = cand[0];
+    if (cand.size() > 1) {
+      CK(timer.run((int)cand.size(), c->st, ms, [&](int q) {
         return launch_lap(L.L.order, L.g, L.B, L.U, (long long)L.L.M * fs, L.F, (long long)L.L.M * fs,
-                          L.alpha_items, nullptr, nullptr, 0, nullptr, sh, c->st);
-      });
-      if (ms < best) { best = ms; pick = sh; }
+                          L.alpha_items, nullptr, nullptr, 0, nullptr, cand[q], c->st);
+      }));
+      L.shape64 = cand[std::min_element(ms.begin(), ms.end()) - ms.begin()];
     }
-    L.shape64 = pick;
     // How far down to fuse the coarse levels: the fused kernel runs on one SM
     // per item, so deep fusion saves launches but can cost FP64 throughput.
     // Time the V-cycle below the first level with N <= 15 for each choice.
@@ -1405,22 +1450,19 @@ static int autotune_T(heat3d_ctx* c, cudaEvent_t e0, cudaEvent_t e1) {
     for (int k = 1; k < L.nmg; ++k)
       if (L.mg[k].N <= kFusedMaxN) { k15 = k; break; }
     if (c->cfg.fuse_coarse && L.L.order != kCompact && k15 > 0) {
-      float bestf = 1e30f;
-      int pickf = kFusedMaxN;
-      for (int fm : {15, 7, 3, 0}) {
-        L.fuse_max = fm;
-        float ms = time_shape(c, e0, e1, [&] {
-          T* cur = nullptr;
-          return vcycle_level<T>(c, L, 0, k15, 0, L.B, nullptr, nullptr, 0, &cur) == HEAT3D_OK
-                     ? cudaSuccess
-                     : cudaErrorUnknown;
-        });
-        if (tune_log())
+      const int depth[] = {15, 7, 3, 0};
+      CK(timer.run(4, c->st, ms, [&](int q) {
+        T* cur = nullptr;
+        L.fuse_max = depth[q];
+        return vcycle_level<T>(c, L, 0, k15, 0, L.B, nullptr, nullptr, 0, &cur) == HEAT3D_OK
+                   ? cudaSuccess
+                   : cudaErrorUnknown;
+      }));
+      if (tune_log())
+        for (int q = 0; q < 4; ++q)
           fprintf(stderr, "tune fuse T%zu order %d below N %d: fuse_max %d: %.4f ms\n", sizeof(T),
-                  L.L.order, L.mg[k15].N, fm, ms);
-        if (ms < bestf) { bestf = ms; pickf = fm; }
-      }
-      L.fuse_max = pickf;
+                  L.L.order, L.mg[k15].N, depth[q], ms[q]);
+      L.fuse_max = depth[std::min_element(ms.begin(), ms.end()) - ms.begin()];
     }
   }
   return HEAT3D_OK;
@@ -1471,12 +1513,9 @@ int h3d_autotune(heat3d_ctx* c) {
   if (all_listed)
     for (int l = 0; l < c->cfg.nlevels; ++l) all_listed = tune_file_lookup(c, c->lv[l], tf) && all_listed;
   if (all_listed) return HEAT3D_OK;
-  EventPair ev;
-  CK(cudaEventCreate(&ev.e0));
-  CK(cudaEventCreate(&ev.e1));
+  ShapeTimer timer;
   const long long l0 = h3d::launches_total();
-  int rc = h3d_tsize(c) == 4 ? autotune_T<float>(c, ev.e0, ev.e1)
-                             : autotune_T<double>(c, ev.e0, ev.e1);
+  int rc = h3d_tsize(c) == 4 ? autotune_T<float>(c, timer) : autotune_T<double>(c, timer);
   h3d::launches_adjust(-(h3d::launches_total() - l0));  // tuning launches are not work
   CK(cudaStreamSynchronize(c->st));
   if (rc == HEAT3D_OK && tf && tf[0])

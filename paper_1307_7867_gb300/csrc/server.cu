@@ -120,6 +120,14 @@ struct heat3d_server {
   Pool pool;  // the admission thread's own
   std::mutex mu;
   std::condition_variable cv_submit, cv_done;
+  // Steps of different groups run side by side; a group's set-up and its first
+  // step run alone (guarded by mu, cv_gate): they load kernels, time launch
+  // shapes and capture graphs, and the driver makes a first use of a kernel
+  // wait until the GPU is idle, which beside busy groups it may not be for a
+  // second.
+  std::condition_variable cv_gate;
+  int stepping = 0, setups = 0;  // steps in flight; set-ups waiting or running
+  bool setting_up = false;
   std::deque<std::shared_ptr<Req>> pending;
   std::map<uint64_t, std::shared_ptr<Req>> all;
   std::map<int, std::unique_ptr<Group>> groups;  // created and released by the admission thread
@@ -129,6 +137,38 @@ struct heat3d_server {
   bool stop = false;
   std::thread worker;
   char err[512] = {0};
+};
+
+// Holds the server's gate for one step, or alone for a set-up.
+class Gate {
+ public:
+  Gate(heat3d_server* s, bool alone) : s_(s), alone_(alone) {
+    std::unique_lock<std::mutex> lk(s_->mu);
+    if (alone_) {
+      s_->setups += 1;
+      s_->cv_gate.wait(lk, [&] { return s_->stepping == 0 && !s_->setting_up; });
+      s_->setting_up = true;
+    } else {
+      s_->cv_gate.wait(lk, [&] { return s_->setups == 0; });
+      s_->stepping += 1;
+    }
+  }
+  ~Gate() {
+    std::lock_guard<std::mutex> lk(s_->mu);
+    if (alone_) {
+      s_->setups -= 1;
+      s_->setting_up = false;
+    } else {
+      s_->stepping -= 1;
+    }
+    s_->cv_gate.notify_all();
+  }
+  Gate(const Gate&) = delete;
+  Gate& operator=(const Gate&) = delete;
+
+ private:
+  heat3d_server* s_;
+  bool alone_;
 };
 
 static int srv_fail(heat3d_server* s, int code, const char* msg) {
@@ -177,10 +217,17 @@ static Group* get_group(heat3d_server* s, int N) {
   size_t need = group_bytes(s, N, &ws);
   char* chunk = s->pool.alloc(need);
   if (!chunk) return nullptr;
+  Gate gate(s, true);
   auto g = std::make_unique<Group>();
   g->N = N;
   g->chunk = chunk;
-  if (cudaStreamCreateWithFlags(&g->st, cudaStreamNonBlocking) != cudaSuccess) {
+  // A small grid's kernels are a few microseconds each; at an equal priority
+  // each would wait for a large grid's blocks, which fill the GPU for up to a
+  // whole kernel.  The smaller the grid, the higher its stream's priority.
+  int lo = 0, hi = 0;
+  cudaDeviceGetStreamPriorityRange(&lo, &hi);
+  const int prio = std::max(hi, lo - (N <= 63 ? 2 : N <= 127 ? 1 : 0));
+  if (cudaStreamCreateWithPriority(&g->st, cudaStreamNonBlocking, prio) != cudaSuccess) {
     s->pool.release(chunk);
     return nullptr;
   }
@@ -336,6 +383,7 @@ static void complete(heat3d_server* s, Group* g, std::vector<std::shared_ptr<Req
 // residents by one time step per round on the group's stream.
 static void group_loop(heat3d_server* s, Group* g) {
   cudaSetDevice(s->cfg.device);
+  bool first = true;
   for (;;) {
     std::deque<std::shared_ptr<Req>> inc;
     {
@@ -343,26 +391,39 @@ static void group_loop(heat3d_server* s, Group* g) {
       g->cv.wait(lk, [&] { return s->stop || g->stop || !g->incoming.empty() || g->active() > 0; });
       if (s->stop) return;
       if (g->stop && g->incoming.empty() && g->active() == 0) return;
-      inc.swap(g->incoming);
+      // An idle group starts with the request that woke it and takes what has
+      // arrived by then in its next round, so that the same submissions make
+      // the same batches (the FP32 cycles per refinement step are chosen for a
+      // batch) however fast this thread wakes.
+      if (g->active() == 0) {
+        inc.push_back(g->incoming.front());
+        g->incoming.pop_front();
+      } else {
+        inc.swap(g->incoming);
+      }
     }
     std::vector<std::shared_ptr<Req>> fin;
-    for (auto& r : inc) {
-      int slot = -1;
-      for (int i = 0; i < (int)g->slots.size(); ++i)
-        if (!g->slots[i]) { slot = i; break; }
-      int rc = slot < 0 ? HEAT3D_EINVAL : admit(s, g, slot, *r);
-      if (rc < 0) {
-        r->status = rc;
-        fin.push_back(r);
-        continue;
+    {
+      Gate gate(s, first);
+      first = false;
+      for (auto& r : inc) {
+        int slot = -1;
+        for (int i = 0; i < (int)g->slots.size(); ++i)
+          if (!g->slots[i]) { slot = i; break; }
+        int rc = slot < 0 ? HEAT3D_EINVAL : admit(s, g, slot, *r);
+        if (rc < 0) {
+          r->status = rc;
+          fin.push_back(r);
+          continue;
+        }
+        g->slots[slot] = r;
       }
-      g->slots[slot] = r;
-    }
-    int rc = step_group(s, g, fin);
-    if (rc < 0) {
-      for (auto& r : g->slots)
-        if (r) { r->status = rc; fin.push_back(r); r->slot = -1; }
-      std::fill(g->slots.begin(), g->slots.end(), nullptr);
+      int rc = step_group(s, g, fin);
+      if (rc < 0) {
+        for (auto& r : g->slots)
+          if (r) { r->status = rc; fin.push_back(r); r->slot = -1; }
+        std::fill(g->slots.begin(), g->slots.end(), nullptr);
+      }
     }
     complete(s, g, fin);
   }
