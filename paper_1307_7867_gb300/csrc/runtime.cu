@@ -1393,13 +1393,14 @@ static std::vector<Shape> shape_candidates(int N, bool vec4) {
       for (int zc : chunks)
         if (zc <= N) v.push_back(Shape{kind, zc});
   };
+  if (!vec4 && N >= kFixMinN) {  // one kernel, which divides the planes itself
+    v.push_back(Shape{kFixKind, 0});
+    return v;
+  }
   add({1}, {1, 2, 4, 8});
   if (N < 16) return v;
   add({2, 4, 5}, {2, 4, 8});
-  if (!vec4) {
-    if (N >= 127) add({3, 4, 5, 6}, {16, 32, 64});
-    return v;
-  }
+  if (!vec4) return v;
   if (N < 127) {
     add({7, 8, 9}, {4, 8});
     add({16, 20, 24}, {8, -1});

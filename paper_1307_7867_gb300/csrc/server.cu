@@ -238,6 +238,12 @@ static Group* get_group(heat3d_server* s, int N) {
     s->pool.release(chunk);
     return nullptr;
   }
+  // its large FP64 kernels leave some of the GPU to the other groups' (the
+  // blocks of 12 SMs of 152)
+  SdcLevel& L = g->ctx->lv[0];
+  if (L.shape64.kind == kFixKind) L.shape64.zc = 24;
+  for (int k = 0; k < L.nmg; ++k)
+    if (L.shapeT[k].kind == kFixKind) L.shapeT[k].zc = 24;
   char* p = chunk + (ws + 255) / 256 * 256;
   Grid gr = make_grid(N);
   g->ucur = (double*)p;

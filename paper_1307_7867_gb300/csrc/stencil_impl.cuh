@@ -19,6 +19,8 @@
 //    with each thread's own points of the planes k-R .. k+R in a register
 //    queue; planes by cp.async or TMA (mbarrier per ring slot), k_zq4p as a
 //    producer/consumer pipeline without block barriers.
+//  * k_fix (stencil_fix.cuh; every FP64 stencil of grids with N >= 127): the
+//    neighbour sums in 64-bit fixed point.
 //  * k_zmarch (small grids): one (x, y) column per thread, z-neighbours in a
 //    register queue, x/y neighbours through L1.
 // Boundary rule of every stencil read: indices -1 and N are the Dirichlet
@@ -102,8 +104,33 @@ __device__ __forceinline__ void warp_max_to(unsigned long long v, unsigned long 
   if ((threadIdx.x & 31) == 0 && v != 0ull) atomicMax(dst, v);
 }
 
+// Centre and neighbour sums of one point straight from the field, in the
+// order of every stencil kernel.
+template <int ORDER>
+__device__ __forceinline__ void plain_sums(const double* __restrict__ u, const Grid& g, int i, int j, int k,
+                                           double& c, double& s1, double& s2) {
+  c = at(u, g, i, j, k);
+  s1 = ((at(u, g, i - 1, j, k) + at(u, g, i + 1, j, k)) + (at(u, g, i, j - 1, k) + at(u, g, i, j + 1, k))) +
+       (at(u, g, i, j, k - 1) + at(u, g, i, j, k + 1));
+  s2 = 0.0;
+  if (ORDER == 4)
+    s2 = ((at(u, g, i - 2, j, k) + at(u, g, i + 2, j, k)) + (at(u, g, i, j - 2, k) + at(u, g, i, j + 2, k))) +
+         (at(u, g, i, j, k - 2) + at(u, g, i, j, k + 2));
+  if (ORDER == kCompact)
+    s2 = (((at(u, g, i - 1, j - 1, k) + at(u, g, i + 1, j - 1, k)) +
+           (at(u, g, i - 1, j + 1, k) + at(u, g, i + 1, j + 1, k))) +
+          ((at(u, g, i - 1, j, k - 1) + at(u, g, i + 1, j, k - 1)) +
+           (at(u, g, i - 1, j, k + 1) + at(u, g, i + 1, j, k + 1)))) +
+         ((at(u, g, i, j - 1, k - 1) + at(u, g, i, j + 1, k - 1)) +
+          (at(u, g, i, j - 1, k + 1) + at(u, g, i, j + 1, k + 1)));
+}
+
 __device__ __forceinline__ void cp_async16(unsigned s, const void* gmem) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
+}
+// As cp_async16, of which the first `bytes` are read and the rest zero.
+__device__ __forceinline__ void cp_async16_fill(unsigned s, const void* gmem, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(s), "l"(gmem), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int n>
@@ -174,9 +201,48 @@ __device__ __forceinline__ T a_res(T d, T e, T e2, T c, T s1, T s2, T b) {
   return fma(-d, c, fma(e, combine<T, ORDER>(s1, s2), b));
 }
 
+}  // namespace
+}  // namespace h3d
+#include "stencil_fix.cuh"
+namespace h3d {
+namespace {
+
+// Two consecutive x points of a row at an even x: n >= 1 of them in the grid.
+__device__ __forceinline__ void store2(double* p, int n, double a, double b) {
+  if (n >= 2) *reinterpret_cast<double2*>(p) = make_double2(a, b);
+  else *p = a;
+}
+__device__ __forceinline__ void store2(float* p, int n, float a, float b) {
+  if (n >= 2) *reinterpret_cast<float2*>(p) = make_float2(a, b);
+  else *p = a;
+}
+
 // ---------------------------------------------------------------------------
 // operators
 // ---------------------------------------------------------------------------
+//
+// fix_init .. put2 serve k_fix (stencil_fix.cuh), two x points at a time:
+// fix_init tells whether the coefficients of the sums may be scaled by their
+// exponent fields, fix_scales scales them to a unit of 2^ke; load2 reads what
+// pre2 needs (the FP64 work without the sums, done while they are formed),
+// late2 what put2 needs; post2 takes the fixed-point sums d1 (7-point: L,
+// wide: L / 16, compact: D1) and d2 (compact: D2) in that unit and put2
+// stores.  In terms of these sums the operators are
+//   A u = c - e L (compact: c - e D1 - e2 D2),
+//   Jacobi  v = (1 - wd) c + be L (compact: + be D1 + be2 D2) + b',
+//   residual t' = b' - wd c + be L (...),
+// the same formulas with d = 1 + 6 e, 1 + 90 e or 1 + 6 e + 12 e2 put in, and
+// with fewer cancelling digits.
+template <int ORDER>
+__device__ constexpr int fix_unit() {  // L in units of d1
+  return ORDER == 4 ? 4 : 0;
+}
+// t + k1 d1 (compact: + k2 d2) for two points
+template <int ORDER>
+__device__ __forceinline__ double2 fix_combine(double2 t, longlong2 d1, longlong2 d2, double k1, double k2) {
+  if (ORDER == kCompact) t = make_double2(fma(k2, fix_double(d2.x), t.x), fma(k2, fix_double(d2.y), t.y));
+  return make_double2(fma(k1, fix_double(d1.x), t.x), fma(k1, fix_double(d1.y), t.y));
+}
 
 // F = alpha_b L u (and, when ADD, the next substep's rhs add_dst = u + add_src).
 // Compact stencil: F = alpha_b (-24 u + 2 S1 + S2) with alpha = nu / (6 h^2);
@@ -227,6 +293,48 @@ struct OpLap {
     if (ADD) ad_[idx] = c + ex.add;
     return 0.0;
   }
+  struct Ex2 { double2 add; };
+  __device__ bool fix_init() const { return fix_coef_ok(a); }
+  __device__ void fix_scales(int ke, double& k1, double& k2) const {
+    k1 = fix_scale(a, ke + (ORDER == kCompact ? 1 : fix_unit<ORDER>()));
+    k2 = fix_scale(1.0 / 12.0, ke);
+  }
+  __device__ Ex2 load2(int idx) const {
+    Ex2 x;
+    if (ADD) x.add = *reinterpret_cast<const double2*>(as_ + idx);
+    return x;
+  }
+  static constexpr bool kFixCentre = ADD || ORDER == kCompact;  // pre2, post2 use the centre
+  struct Pre { double2 t; };                // W u + add without D1
+  struct Out2 { double2 f, w, a; };
+  struct Late {};
+  __device__ Late late2(int) const { return Late{}; }
+  __device__ Pre pre2(double2 c, const Ex2& ex) const {
+    Pre p;
+    if (ADD) p.t = make_double2(c.x + ex.add.x, c.y + ex.add.y);
+    return p;
+  }
+  __device__ Out2 post2(const Pre& p, double2 c, longlong2 d1, longlong2 d2, double k1, double k2) const {
+    Out2 o;
+    if (ORDER == kCompact) {  // L = 2 (D1 + D2 / 2); W u = c + D1 / 12
+      o.f = make_double2(k1 * fix_double(d1.x + (d2.x >> 1)), k1 * fix_double(d1.y + (d2.y >> 1)));
+      if (wu_ || ADD) {
+        const double w0 = fix_double(d1.x), w1 = fix_double(d1.y);
+        o.w = make_double2(fma(k2, w0, c.x), fma(k2, w1, c.y));
+        if (ADD) o.a = make_double2(fma(k2, w0, p.t.x), fma(k2, w1, p.t.y));
+      }
+    } else {
+      o.f = make_double2(k1 * fix_double(d1.x), k1 * fix_double(d1.y));
+      if (ADD) o.a = p.t;
+    }
+    return o;
+  }
+  template <bool NORM>
+  __device__ void put2(int idx, int n, const Out2& o, const Late&, unsigned long long&) {
+    store2(o_ + idx, n, o.f.x, o.f.y);
+    if (ORDER == kCompact && wu_) store2(wu_ + idx, n, o.w.x, o.w.y);
+    if (ADD) store2(ad_ + idx, n, o.a.x, o.a.y);
+  }
 };
 
 // r = b - A u in FP64 (its max |.| is the stop rule's norm), stored as the
@@ -258,6 +366,27 @@ struct OpResid64 {
     double res = a_res<double, ORDER>(d, e, e2, c, s1, s2, ex.b);
     bp_[idx] = wd * (TR)res;
     return res;
+  }
+  struct Ex2 { double2 b; };
+  __device__ bool fix_init() const { return fix_coef_ok(e) && fix_coef_ok(e2); }
+  __device__ void fix_scales(int ke, double& k1, double& k2) const {
+    k1 = fix_scale(e, ke + fix_unit<ORDER>());
+    k2 = fix_scale(e2, ke);
+  }
+  __device__ Ex2 load2(int idx) const { return Ex2{*reinterpret_cast<const double2*>(b_ + idx)}; }
+  static constexpr bool kFixCentre = true;
+  struct Pre { double2 t; };  // b - c
+  struct Out2 { double2 r; };
+  struct Late {};
+  __device__ Late late2(int) const { return Late{}; }
+  __device__ Pre pre2(double2 c, const Ex2& ex) const { return Pre{make_double2(ex.b.x - c.x, ex.b.y - c.y)}; }
+  __device__ Out2 post2(const Pre& p, double2, longlong2 d1, longlong2 d2, double k1, double k2) const {
+    return Out2{fix_combine<ORDER>(p.t, d1, d2, k1, k2)};
+  }
+  template <bool NORM>
+  __device__ void put2(int idx, int n, const Out2& o, const Late&, unsigned long long& mx) {
+    store2(bp_ + idx, n, wd * (TR)o.r.x, wd * (TR)o.r.y);
+    if (NORM) mx = max(mx, max(abs_bits(o.r.x), n >= 2 ? abs_bits(o.r.y) : 0ull));
   }
 };
 
@@ -299,6 +428,7 @@ struct OpJacobi {
     al = coef[b].al;
     be = coef[b].be;
     be2 = coef[b].be2;
+    if (sizeof(T) == 8) w1_ = 1.0 - coef[b].wd;
     r_ = r + b * fs;
     if (UPD) u_ = u64 + b * u64s;
     else o_ = out + b * fs;
@@ -314,6 +444,34 @@ struct OpJacobi {
     if (UPD) u_[idx] = ex.u + (double)v;
     else o_[idx] = v;
     return 0.0;
+  }
+  double w1_;  // 1 - wd
+  struct Ex2 { double2 r; };
+  struct Late { double2 u; };
+  static constexpr bool kFixCentre = true;
+  struct Pre { double2 t; };  // (1 - wd) c + b'
+  struct Out2 { double2 v; };
+  __device__ bool fix_init() const { return fix_coef_ok(be) && fix_coef_ok(be2); }
+  __device__ void fix_scales(int ke, double& k1, double& k2) const {
+    k1 = fix_scale(be, ke + fix_unit<ORDER>());
+    k2 = fix_scale(be2, ke);
+  }
+  __device__ Ex2 load2(int idx) const { return Ex2{*reinterpret_cast<const double2*>(r_ + idx)}; }
+  __device__ Late late2(int idx) const {
+    Late l;
+    if (UPD) l.u = *reinterpret_cast<const double2*>(u_ + idx);
+    return l;
+  }
+  __device__ Pre pre2(double2 c, const Ex2& ex) const {
+    return Pre{make_double2(fma(w1_, c.x, ex.r.x), fma(w1_, c.y, ex.r.y))};
+  }
+  __device__ Out2 post2(const Pre& p, double2, longlong2 d1, longlong2 d2, double k1, double k2) const {
+    return Out2{fix_combine<ORDER>(p.t, d1, d2, k1, k2)};
+  }
+  template <bool NORM>
+  __device__ void put2(int idx, int n, const Out2& o, const Late& l, unsigned long long&) {
+    if (UPD) store2(u_ + idx, n, l.u.x + o.v.x, l.u.y + o.v.y);
+    else store2(o_ + idx, n, o.v.x, o.v.y);
   }
   // Four consecutive x points (FP32 storage, k_tile4): idx is a multiple of
   // 4, n >= 1 of the four are inside the grid.  Same arithmetic per point as
@@ -376,6 +534,7 @@ struct OpResid {
     om = coef[b].om;
     be = coef[b].be;
     be2 = coef[b].be2;
+    if (sizeof(T) == 8) wd = coef[b].wd;
     r_ = r + b * fs;
     o_ = rr + b * fs;
   }
@@ -383,6 +542,29 @@ struct OpResid {
   __device__ double apply(int idx, T c, T s1, T s2, const Ex& ex) {
     o_[idx] = resid_point<T, ORDER>(om, be, be2, c, s1, s2, ex.r);
     return 0.0;
+  }
+  double wd;
+  struct Ex2 { double2 r; };
+  __device__ bool fix_init() const { return fix_coef_ok(be) && fix_coef_ok(be2); }
+  __device__ void fix_scales(int ke, double& k1, double& k2) const {
+    k1 = fix_scale(be, ke + fix_unit<ORDER>());
+    k2 = fix_scale(be2, ke);
+  }
+  __device__ Ex2 load2(int idx) const { return Ex2{*reinterpret_cast<const double2*>(r_ + idx)}; }
+  struct Late {};
+  static constexpr bool kFixCentre = true;
+  struct Pre { double2 t; };  // b' - wd c
+  struct Out2 { double2 v; };
+  __device__ Late late2(int) const { return Late{}; }
+  __device__ Pre pre2(double2 c, const Ex2& ex) const {
+    return Pre{make_double2(fma(-wd, c.x, ex.r.x), fma(-wd, c.y, ex.r.y))};
+  }
+  __device__ Out2 post2(const Pre& p, double2, longlong2 d1, longlong2 d2, double k1, double k2) const {
+    return Out2{fix_combine<ORDER>(p.t, d1, d2, k1, k2)};
+  }
+  template <bool NORM>
+  __device__ void put2(int idx, int n, const Out2& o, const Late&, unsigned long long&) {
+    store2(o_ + idx, n, o.v.x, o.v.y);
   }
   static constexpr bool kVec4 = sizeof(TT) == 4;
   static constexpr int kRegFloor = ORDER == kCompact ? 128 : 64;
@@ -1489,6 +1671,14 @@ cudaError_t run_stencil(const Grid& g, int B, const int* active, unsigned long l
                         const Op& op, Shape sh, cudaStream_t st) {
   if (B <= 0 || g.N <= 0) return cudaSuccess;
   int kind = sh.kind;
+  if constexpr (sizeof(typename Op::T) == 8) {
+    if (g.N >= kFixMinN) {
+      cudaError_t e = launch_fix<ORDER, NORM>(g, B, kind == kFixKind ? sh.zc : 0, active, norm_bits, op, st);
+      if (e != cudaSuccess) return e;
+      count_launch();
+      return cudaGetLastError();
+    }
+  }
   if (kind == 0) kind = g.N >= 32 ? 3 : 1;
   int zc = sh.zc > 0 ? sh.zc : 16;
   if (zc > g.N) zc = g.N;
