@@ -8,6 +8,7 @@
 // requests, nodes) follow each other at the field stride fs.
 #pragma once
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 namespace h3d {
@@ -113,7 +114,59 @@ struct ItemSDC {
   double dtQ[kMaxNodes][kMaxNodes];      // dt * Q[m][j]  (FAS restriction, fine level)
   double gQ[kMaxNodes];                  // dt * sum_j Q[m][j] g(t0 + dt tau_j)
   double nu;
+  // the quadrature kernel's two matrices in fixed point (fix_coefficients),
+  // value = (x 2^31 + y) 2^(fe - 59), |y| <= 2^30: rows of the substep
+  // integrals I_m (dtS with -dtm on F_{m+1}) and of the partial sums of J;
+  // column M: the forcing, for the field 2^fp Phi, which has the size of the
+  // forcing against F (forced = 0: none).  fok = 0: they do not fit the format.
+  int2 fI[kMaxNodes - 1][kMaxNodes + 1];
+  int2 fQ[kMaxNodes - 1][kMaxNodes + 1];
+  int fe, fok, fp, forced;
 };
+
+// The fixed-point copies: fe is such that the sum of magnitudes of every row
+// of both matrices is below 2^fe.
+inline void fix_coefficients(ItemSDC& it, int M) {
+  double gmax = 0.0, smax = 0.0;
+  for (int m = 0; m + 1 < M; ++m) {
+    gmax = fmax(gmax, fabs(it.gS[m]));
+    for (int j = 0; j < M; ++j) smax = fmax(smax, fabs(it.dtS[m][j]));
+  }
+  it.forced = gmax > 0.0;
+  it.fp = it.forced ? ilogb(gmax) - ilogb(smax) : 0;
+  auto g = [&](int m) { return ldexp(it.gS[m], -it.fp); };
+  double s = 0.0, cs[kMaxNodes + 1] = {0.0};
+  for (int m = 0; m + 1 < M; ++m) {
+    double ri = it.dtm[m], rq = 0.0;
+    for (int j = 0; j <= M; ++j) {
+      const double v = j < M ? it.dtS[m][j] : g(m);
+      cs[j] += v;
+      ri += fabs(v);
+      rq += fabs(cs[j]);
+    }
+    s = fmax(s, fmax(ri, rq));
+  }
+  s *= 1.0 + 1e-9;  // over the copies' own rounding
+  it.fok = s > 1e-60 && s < 1e60 && it.fp > -200 && it.fp < 200;
+  it.fe = 0;
+  if (!it.fok) return;
+  double scale = 576460752303423488.0;  // 2^59
+  while (s >= 1.0) { s *= 0.5; scale *= 0.5; it.fe += 1; }
+  while (s < 0.5) { s *= 2.0; scale *= 2.0; it.fe -= 1; }
+  auto fixed = [&](double c) { return (long long)(c * scale + (c < 0 ? -0.5 : 0.5)); };
+  auto split = [](long long v) {
+    const long long hi = (v + (1ll << 30)) >> 31;
+    return make_int2((int)hi, (int)(v - hi * (1ll << 31)));
+  };
+  long long cum[kMaxNodes + 1] = {0};
+  for (int m = 0; m + 1 < M; ++m)
+    for (int j = 0; j <= M; ++j) {
+      const long long v = fixed(j < M ? it.dtS[m][j] : g(m));
+      cum[j] += v;
+      it.fI[m][j] = split(j == m + 1 ? v - fixed(it.dtm[m]) : v);
+      it.fQ[m][j] = split(cum[j]);
+    }
+}
 
 // FAS transfer data between the fine (F) and coarse (G) levels.
 struct FasMap {

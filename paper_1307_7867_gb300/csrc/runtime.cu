@@ -359,6 +359,7 @@ void h3d_fill_item(heat3d_ctx* c, int lev, int item, double t0) {
     }
     it.gQ[m] = s;
   }
+  fix_coefficients(it, M);
   L.t0[item] = t0;
 }
 

@@ -1,5 +1,8 @@
-// sdc_kernels.cu -- spectral-quadrature and FAS kernels (Sec. 1.1).
-// All are point-parallel: one thread per grid point of one item, FP64.
+// sdc_kernels.cu -- spectral-quadrature and FAS kernels (Sec. 1.1), point by
+// point; the quadrature sums in fixed point, everything else FP64.
+#include <type_traits>
+
+#include "fix.cuh"
 #include "kernels.cuh"
 
 namespace h3d {
@@ -24,49 +27,167 @@ inline dim3 point_grid(const Grid& g, int B) {
 
 // Quadrature integrals of one sweep and (optionally) the collocation residual
 // of the current iterate.  I == nullptr: residual only.
+//
+// With FP64 multiply-adds a point costs 43 FP64 operations (M = 5), 1.40 ms at
+// 255^3 on a pipe of 2 per clock and SM, five times the memory time of its
+// 10 to 14 fields.  The sums run in fixed point instead: the F values of a
+// point (and Phi, scaled by a power of two
+// to the size of the forcing) are brought to the largest exponent among them, 59 bits of
+// each multiplied with 59-bit copies of the matrices (ItemSDC::fI, fQ) as two
+// centred 31-bit digits, and each sum becomes a double once.  Points whose exponents the format does not take go through FP64
+// (plain).  A thread takes a run of kz points along z, which shares the loads
+// of the digits and phi_x phi_y.
+struct FixTerm {
+  int h, l;
+};
+__device__ __forceinline__ FixTerm fix_digits(double x, int E) {
+  const long long v = fix_value<6>(__double2hiint(x), __double2loint(x), E);
+  const int h = (int)((v + (1ll << 30)) >> 31);
+  return FixTerm{h, (int)(unsigned)v - (int)((unsigned)h << 31)};
+}
+// Sum of products in three parts: 2^62 hi + 2^31 mid + 2^32 lo.
+struct FixSum {
+  long long hi = 0, mid = 0;
+  int lo = 0;
+  __device__ void add(FixTerm f, int2 c) {
+    hi += (long long)f.h * c.x;
+    mid += (long long)f.h * c.y;
+    mid += (long long)f.l * c.x;
+    lo += __mulhi(f.l, c.y);
+  }
+  __device__ long long value() const { return (hi << 6) + ((mid + 2 * lo) >> 25); }  // of 2^56
+};
+
+// The FP64 form of one point (also the reading of the sums: J_m, I_m, r_m).
 template <int M>
-__global__ void k_integrals(Grid g, const double* __restrict__ U, const double* __restrict__ F,
-                            const double* __restrict__ tauS, double* __restrict__ I,
-                            const ItemSDC* __restrict__ items, const double* __restrict__ phi1d,
-                            unsigned long long* res_bits, const int* active) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  const int b = blockIdx.z / g.N;
-  const int k = blockIdx.z - b * g.N;
-  if (active && !active[b]) return;  // uniform over the block
+__device__ __noinline__ unsigned long long integrals_plain(const ItemSDC& it, const double* Ub, const double* Fb,
+                                                           const double* tb, double* Ib, long long fs, double phi,
+                                                           bool res) {
+  const double u0 = Ub[0];
+  double cum = 0.0;
   unsigned long long mx = 0ull;
-  if (i < g.N && j < g.N) {
-    const long long idx = (long long)k * g.plane + (long long)j * g.px + i;
-    const long long fs = g.fs;
-    const double* Ub = U + (long long)b * M * fs + idx;
-    const double* Fb = F + (long long)b * M * fs + idx;
-    const ItemSDC& it = items[b];
-    double Fj[M];
-#pragma unroll
-    for (int q = 0; q < M; ++q) Fj[q] = Fb[q * fs];
-    const double phi = phi1d[i] * phi1d[j] * phi1d[k];
-    const double u0 = Ub[0];
-    double cum = 0.0;
-#pragma unroll
-    for (int m = 0; m < M - 1; ++m) {
-      double J = it.gS[m] * phi;
-#pragma unroll
-      for (int q = 0; q < M; ++q) J = fma(it.dtS[m][q], Fj[q], J);
-      if (tauS) J += tauS[((long long)b * (M - 1) + m) * fs + idx];
-      if (I) {
-        double Im = fma(-it.dtm[m], Fj[m + 1], J);
-        if (m == 0) Im += u0;
-        I[((long long)b * (M - 1) + m) * fs + idx] = Im;
-      }
-      if (res_bits) {
-        cum += J;
-        double rv = (u0 + cum) - Ub[(m + 1) * fs];
-        unsigned long long bits = abs_bits(rv);
-        mx = bits > mx ? bits : mx;
-      }
+  for (int m = 0; m < M - 1; ++m) {
+    double J = it.gS[m] * phi;
+    for (int q = 0; q < M; ++q) J = fma(it.dtS[m][q], Fb[q * fs], J);
+    if (tb) J += tb[m * fs];
+    if (Ib) {
+      double Im = fma(-it.dtm[m], Fb[(m + 1) * fs], J);
+      if (m == 0) Im += u0;
+      Ib[m * fs] = Im;
+    }
+    if (res) {
+      cum += J;
+      const unsigned long long bits = abs_bits((u0 + cum) - Ub[(m + 1) * fs]);
+      mx = bits > mx ? bits : mx;
     }
   }
-  if (res_bits) warp_max_to(mx, res_bits + b);
+  return mx;
+}
+
+template <int M, bool TAU, bool RES>
+__global__ void __launch_bounds__(256, 4) k_integrals(Grid g, const double* __restrict__ U,
+                                                      const double* __restrict__ F,
+                                                      const double* __restrict__ tauS,
+                                                      double* __restrict__ I,
+                                                      const ItemSDC* __restrict__ items,
+                                                      const double* __restrict__ phi1d,
+                                                      unsigned long long* res_bits, const int* active,
+                                                      int kz) {
+  constexpr int C = (M + 2) / 2 * 2;  // columns, an even number
+  __shared__ __align__(16) int2 cI[M - 1][C], cQ[M - 1][C];
+  const int nkz = (g.N + kz - 1) / kz;
+  const int b = blockIdx.z / nkz;
+  if (active && !active[b]) return;  // uniform over the block
+  const ItemSDC& it = items[b];
+  const int tid = threadIdx.y * 32 + threadIdx.x;
+  if (tid < (M - 1) * C) {
+    const int m = tid / C, j = tid - m * C;
+    cI[m][j] = j <= M ? it.fI[m][j] : make_int2(0, 0);
+    cQ[m][j] = j <= M ? it.fQ[m][j] : make_int2(0, 0);
+  }
+  const int fe = it.fe, fp = it.fp;
+  const bool forced = it.forced != 0;
+  const bool fok = it.fok != 0;
+  __syncthreads();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = blockIdx.y * blockDim.y + threadIdx.y;
+  const int k0 = (blockIdx.z - b * nkz) * kz, k1 = min(g.N, k0 + kz);
+  unsigned long long mx = 0ull;
+  if (i < g.N && j < g.N) {
+    const long long fs = g.fs;
+    const double phixy = phi1d[i] * phi1d[j];
+#pragma unroll 1
+    for (int k = k0; k < k1; ++k) {
+      const long long idx = (long long)k * g.plane + (long long)j * g.px + i;
+      const double* Ub = U + (long long)b * M * fs + idx;
+      const double* Fb = F + (long long)b * M * fs + idx;
+      const double* tb = TAU ? tauS + (long long)b * (M - 1) * fs + idx : nullptr;
+      double* Ib = I ? I + (long long)b * (M - 1) * fs + idx : nullptr;
+      const double phi = phixy * phi1d[k];
+      FixTerm f[C];
+      int E;
+      {
+        double x[C];
+        unsigned key = 0u;
+#pragma unroll
+        for (int q = 0; q < C; ++q) {
+          x[q] = q < M ? Fb[q * fs] : q == M && forced ? fix_scale(phi, fp) : 0.0;
+          key = max(key, (unsigned)__double2hiint(x[q]) & 0x7fffffffu);
+        }
+        E = fix_exponent(key);
+#pragma unroll
+        for (int q = 0; q < C; ++q) f[q] = q <= M ? fix_digits(x[q], E) : FixTerm{0, 0};
+      }
+      if (!fok || E > kFixHi || (E < kFixLo && E != kFixZero)) {
+        const unsigned long long bits = integrals_plain<M>(it, Ub, Fb, tb, Ib, fs, phi, RES);
+        mx = bits > mx ? bits : mx;
+        continue;
+      }
+      const int ke = E - 1084 + fe;
+      auto row = [&](const int2* c) {  // one row's sum as a double
+        FixSum s;
+#pragma unroll
+        for (int q = 0; q < C; q += 2) {
+          const int4 v = *reinterpret_cast<const int4*>(c + q);
+          s.add(f[q], make_int2(v.x, v.y));
+          if (q + 1 <= M) s.add(f[q + 1], make_int2(v.z, v.w));
+        }
+        return fix_scale(fix_double(s.value()), ke);
+      };
+      const double u0 = Ub[0];
+      double ctau = 0.0;
+      // row m; the one that adds U_0 stands apart (an FP64 addition under a
+      // condition runs for every row)
+      auto substep = [&](int m, auto first) {
+        const double tau = TAU ? tb[m * fs] : 0.0;
+        if (I) {
+          double Im = row(cI[m]);
+          if (TAU) Im += tau;
+          if (decltype(first)::value) Im += u0;
+          Ib[m * fs] = Im;
+        }
+        if (RES) {
+          double rv = (u0 - Ub[(m + 1) * fs]) + row(cQ[m]);
+          if (TAU) rv += ctau += tau;
+          const unsigned long long bits = abs_bits(rv);
+          mx = bits > mx ? bits : mx;
+        }
+      };
+      substep(0, std::true_type{});
+#pragma unroll 1
+      for (int m = 1; m < M - 1; ++m) substep(m, std::false_type{});
+    }
+  }
+  if (RES) warp_max_to(mx, res_bits + b);
+}
+
+template <int M>
+void start_integrals(dim3 grd, dim3 blk, cudaStream_t st, const Grid& g, const double* U, const double* F,
+                     const double* tauS, double* I, const ItemSDC* items, const double* phi1d,
+                     unsigned long long* res_bits, const int* active, int kz) {
+  auto k = tauS ? (res_bits ? k_integrals<M, true, true> : k_integrals<M, true, false>)
+                : (res_bits ? k_integrals<M, false, true> : k_integrals<M, false, false>);
+  k<<<grd, blk, 0, st>>>(g, U, F, tauS, I, items, phi1d, res_bits, active, kz);
 }
 
 // Coarse point (I, J, K) (0-based) sits on fine point (2I+1, 2J+1, 2K+1), or on
@@ -201,12 +322,14 @@ cudaError_t launch_integrals(int M, const Grid& g, int B, const double* U, const
                              const double* phi1d, unsigned long long* res_bits,
                              const int* active, cudaStream_t st) {
   if (B <= 0) return cudaSuccess;
-  dim3 grd = point_grid(g, B), blk(32, 8);
+  // points per thread: as many as leave several blocks for every SM
+  const int kz = g.N >= 255 ? 8 : g.N >= 127 ? 4 : 1;
+  const dim3 grd((g.N + 31) / 32, (g.N + 7) / 8, (g.N + kz - 1) / kz * B), blk(32, 8);
   switch (M) {
-    case 2: k_integrals<2><<<grd, blk, 0, st>>>(g, U, F, tauS, I, items, phi1d, res_bits, active); break;
-    case 3: k_integrals<3><<<grd, blk, 0, st>>>(g, U, F, tauS, I, items, phi1d, res_bits, active); break;
-    case 4: k_integrals<4><<<grd, blk, 0, st>>>(g, U, F, tauS, I, items, phi1d, res_bits, active); break;
-    case 5: k_integrals<5><<<grd, blk, 0, st>>>(g, U, F, tauS, I, items, phi1d, res_bits, active); break;
+    case 2: start_integrals<2>(grd, blk, st, g, U, F, tauS, I, items, phi1d, res_bits, active, kz); break;
+    case 3: start_integrals<3>(grd, blk, st, g, U, F, tauS, I, items, phi1d, res_bits, active, kz); break;
+    case 4: start_integrals<4>(grd, blk, st, g, U, F, tauS, I, items, phi1d, res_bits, active, kz); break;
+    case 5: start_integrals<5>(grd, blk, st, g, U, F, tauS, I, items, phi1d, res_bits, active, kz); break;
     default: return cudaErrorInvalidValue;
   }
   count_launch();
