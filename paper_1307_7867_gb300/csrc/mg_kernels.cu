@@ -1,8 +1,8 @@
 // mg_kernels.cu -- point-parallel multigrid and layout kernels (Sec. 1.2):
 // Jacobi from a zero initial guess and the exact one-unknown solve, full
 // weighting restriction, trilinear prolongation, the FP64 update, max-norms
-// and the dense <-> pitched copies.  One thread per grid point of one item;
-// blockIdx.z = item * N + plane.  (The stencil kernels are in
+// and the dense <-> pitched copies.  One thread per grid point of one item
+// (blockIdx.z = item * N + plane) but for the copies.  (The stencil kernels are in
 // stencil_impl.cuh.)
 #include <algorithm>
 
@@ -398,27 +398,57 @@ __global__ void k_maxabs(Grid g, const double* __restrict__ u, long long us,
   warp_max_to(v, norm_bits + b);
 }
 
-__global__ void k_dense_to_pitched(Grid g, const double* __restrict__ d, double* __restrict__ f,
-                                   long long fsd) {
-  PointIdx p;
-  if (!point_index(g, p)) return;
-  long long n = (long long)g.N;
-  f[p.b * fsd + p.idx] = d[((p.b * n + p.k) * n + p.j) * n + p.i];
+// Layout and copy kernels: memory bound, so a thread moves several planes with
+// all its loads in flight before the first store (one value per thread left
+// about a third of the bandwidth in use: 16 KB in flight on an SM).
+constexpr int kMoveZ = 8;
+
+inline dim3 move_grid(const Grid& g, int nx, int B) {
+  return dim3((nx + 31) / 32, (g.N + 7) / 8, (g.N + kMoveZ - 1) / kMoveZ * B);
 }
 
-__global__ void k_pitched_to_dense(Grid g, const double* __restrict__ f, long long fsd,
-                                   double* __restrict__ d) {
-  PointIdx p;
-  if (!point_index(g, p)) return;
-  long long n = (long long)g.N;
-  d[((p.b * n + p.k) * n + p.j) * n + p.i] = f[p.b * fsd + p.idx];
+// dense rows have no alignment beyond 8 bytes: single values
+template <bool kToPitched>
+__global__ void __launch_bounds__(256) k_dense(Grid g, const double* __restrict__ src,
+                                               double* __restrict__ dst, long long fsd) {
+  const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y;
+  const int nz = (g.N + kMoveZ - 1) / kMoveZ, b = blockIdx.z / nz, k0 = (blockIdx.z - b * nz) * kMoveZ;
+  if (i >= g.N || j >= g.N) return;
+  const long long n = g.N, dn = n * n;
+  const long long dense = ((b * n + k0) * n + j) * n + i;
+  const long long pitched = b * fsd + (long long)k0 * g.plane + (long long)j * g.px + i;
+  const long long so = kToPitched ? dense : pitched, ss = kToPitched ? dn : g.plane;
+  const long long to = kToPitched ? pitched : dense, ts = kToPitched ? g.plane : dn;
+  double v[kMoveZ];
+#pragma unroll
+  for (int q = 0; q < kMoveZ; ++q)
+    if (k0 + q < g.N) v[q] = src[so + q * ss];
+#pragma unroll
+  for (int q = 0; q < kMoveZ; ++q)
+    if (k0 + q < g.N) dst[to + q * ts] = v[q];
 }
 
-__global__ void k_copy(Grid g, const double* __restrict__ s, long long ss, double* __restrict__ d,
-                       long long ds) {
-  PointIdx p;
-  if (!point_index(g, p)) return;
-  d[p.b * ds + p.idx] = s[p.b * ss + p.idx];
+// Item b of the source into nd fields of the destination: two x points a
+// thread (rows are 16-byte aligned; the pad column is read, never written).
+__global__ void __launch_bounds__(256) k_copy(Grid g, int nd, const double* __restrict__ s, long long ss,
+                                              double* __restrict__ d, long long ds) {
+  const int i = 2 * (blockIdx.x * 32 + threadIdx.x), j = blockIdx.y * 8 + threadIdx.y;
+  const int nz = (g.N + kMoveZ - 1) / kMoveZ, b = blockIdx.z / nz, k0 = (blockIdx.z - b * nz) * kMoveZ;
+  if (i >= g.N || j >= g.N) return;
+  const long long o = (long long)k0 * g.plane + (long long)j * g.px + i;
+  double2 v[kMoveZ];
+#pragma unroll
+  for (int q = 0; q < kMoveZ; ++q)
+    if (k0 + q < g.N) v[q] = *reinterpret_cast<const double2*>(s + b * ss + o + q * g.plane);
+  for (int t = 0; t < nd; ++t) {
+    double* p = d + (long long)(b + t) * ds + o;
+#pragma unroll
+    for (int q = 0; q < kMoveZ; ++q) {
+      if (k0 + q >= g.N) continue;
+      if (i + 1 < g.N) *reinterpret_cast<double2*>(p + q * g.plane) = v[q];
+      else p[q * g.plane] = v[q].x;
+    }
+  }
 }
 
 }  // namespace
@@ -545,7 +575,7 @@ cudaError_t launch_maxabs(const Grid& g, int B, const double* u, long long u_str
 cudaError_t launch_dense_to_pitched(const Grid& g, int B, const double* dense, double* f,
                                     long long f_stride, cudaStream_t st) {
   if (B <= 0) return cudaSuccess;
-  k_dense_to_pitched<<<point_grid(g, B), dim3(32, 8), 0, st>>>(g, dense, f, f_stride);
+  k_dense<true><<<move_grid(g, g.N, B), dim3(32, 8), 0, st>>>(g, dense, f, f_stride);
   count_launch();
   return cudaGetLastError();
 }
@@ -553,7 +583,7 @@ cudaError_t launch_dense_to_pitched(const Grid& g, int B, const double* dense, d
 cudaError_t launch_pitched_to_dense(const Grid& g, int B, const double* f, long long f_stride,
                                     double* dense, cudaStream_t st) {
   if (B <= 0) return cudaSuccess;
-  k_pitched_to_dense<<<point_grid(g, B), dim3(32, 8), 0, st>>>(g, f, f_stride, dense);
+  k_dense<false><<<move_grid(g, g.N, B), dim3(32, 8), 0, st>>>(g, f, dense, f_stride);
   count_launch();
   return cudaGetLastError();
 }
@@ -561,7 +591,9 @@ cudaError_t launch_pitched_to_dense(const Grid& g, int B, const double* f, long 
 cudaError_t launch_copy(const Grid& g, int B, const double* src, long long src_stride,
                         double* dst, long long dst_stride, cudaStream_t st) {
   if (B <= 0) return cudaSuccess;
-  k_copy<<<point_grid(g, B), dim3(32, 8), 0, st>>>(g, src, src_stride, dst, dst_stride);
+  // one source field for all items: read once
+  const int nd = src_stride == 0 ? B : 1;
+  k_copy<<<move_grid(g, (g.N + 1) / 2, B / nd), dim3(32, 8), 0, st>>>(g, nd, src, src_stride, dst, dst_stride);
   count_launch();
   return cudaGetLastError();
 }

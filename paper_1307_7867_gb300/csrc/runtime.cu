@@ -1197,12 +1197,26 @@ int h3d_fas_interpolate(heat3d_ctx* c, int b0, int B) {
 // ---------------------------------------------------------------------------
 
 // Spread the pitched field u (one item) to every node of items [b0, b0+B).
+// Their fields are all equal, so the operator is evaluated once (items of one
+// diffusion coefficient) and its result spread like u.
 int h3d_spread(heat3d_ctx* c, int lev, int b0, int B, const double* u) {
   SdcLevel& L = c->lv[lev];
   const int M = L.L.M;
   const long long fs = L.g.fs;
-  CK(launch_copy(L.g, B * M, u, 0, L.U + (size_t)b0 * M * fs, fs, c->st));
-  RET(h3d_eval_F(c, lev, b0, B));
+  double* U = L.U + (size_t)b0 * M * fs;
+  double* F = L.F + (size_t)b0 * M * fs;
+  CK(launch_copy(L.g, B * M, u, 0, U, fs, c->st));
+  bool same = B * M > 1;
+  for (int b = 1; b < B; ++b) same = same && L.nu[b0 + b] == L.nu[b0];
+  if (!same) {
+    RET(h3d_eval_F(c, lev, b0, B));
+  } else {
+    CK(launch_lap(L.L.order, L.g, 1, U, fs, F, fs, L.alpha_items + b0, nullptr, nullptr, 0, nullptr, L.shape64,
+                  c->st, wu_of(L, U)));
+    CK(launch_copy(L.g, B * M - 1, F, 0, F + fs, fs, c->st));
+    if (L.WU) CK(launch_copy(L.g, B * M - 1, wu_of(L, U), 0, wu_of(L, U) + fs, fs, c->st));
+    c->bytes += (16.0 + 8.0 * (B * M - 1)) * L.L.N * L.L.N * (double)L.L.N;
+  }
   c->bytes += 8.0 * L.L.N * L.L.N * (double)L.L.N * B * M;
   return HEAT3D_OK;
 }
