@@ -112,7 +112,8 @@ typedef struct {
                                The environment variable HEAT3D_SHAPE="kind,zc" (kind 1-26,
                                planes per block zc, or -1 / -2 for the chunk that fills one /
                                two waves of the GPU) forces one shape on every stencil of
-                               grids with N >= 16 instead (testing); HEAT3D_TUNE_FILE=path
+                               grids with N >= 16 instead (testing; the FP64 stencils of large
+                               grids have one kernel whatever the shape); HEAT3D_TUNE_FILE=path
                                reuses the shapes recorded in that file for levels it lists
                                and appends the timed choices of the others */
   int fuse_coarse;          /* 1: run the coarse multigrid levels of a V-cycle in one kernel,

@@ -18,10 +18,11 @@ namespace h3d {
 // 2 rows), 11 and 12 as 7 and 8 with 6 planes of prefetch, 13 as 7 with 10,
 // 14 (2 warps x 2 rows, 6 planes); other operators take kind 3 for these; zc:
 // planes per block along z.
-// FP64 stencils on grids with N >= kFixMinN have one kernel (stencil_fix.cuh)
+// FP64 stencils on grids with N >= fix_min_n have one kernel (stencil_fix.cuh)
 // whatever the kind; for kind kFixKind zc is the number of resident blocks
 // that its launches leave to other streams.
-constexpr int kFixMinN = 127, kFixKind = 27;
+constexpr int kFixKind = 27;
+__host__ __device__ constexpr int fix_min_n(int order) { return order == kCompact ? 63 : 127; }
 struct Shape {
   int kind = 0;
   int zc = 16;

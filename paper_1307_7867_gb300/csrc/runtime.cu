@@ -463,10 +463,12 @@ static const Coef<T>* coefT(SdcLevel& L, int slot, int k, int b0) {
 // operations, flops); `upd` adds the result to the FP64 solution; `same`: the
 // iterate is b' itself (the sweep after the one from zero), read once.
 template <typename T>
-static void jacobi_cost(int order, bool upd, bool same, double* bytes, double* dp, double* fl) {
+static void jacobi_cost(int order, int N, bool upd, bool same, double* bytes, double* dp, double* fl) {
   const double ts = sizeof(T);
-  // neighbour sums + fused multiply-adds (an FMA counts 2 flops)
-  const double ops = order == 2 ? 7.0 : order == 4 ? 13.0 : 19.0;
+  // neighbour sums + fused multiply-adds (an FMA counts 2 flops); large grids
+  // form the sums in integers
+  const double ops = N >= fix_min_n(order) ? (order == kCompact ? 3.0 : 2.0)
+                                           : order == 2 ? 7.0 : order == 4 ? 13.0 : 19.0;
   const double flops = order == 2 ? 9.0 : order == 4 ? 16.0 : 22.0;
   *bytes = (upd ? ts + 16.0 : 2.0 * ts) + (same ? 0.0 : ts);
   *dp = (sizeof(T) == 8 ? ops : 0.0) + (upd ? 1.0 : 0.0);
@@ -543,7 +545,7 @@ static int vcycle_level(heat3d_ctx* c, SdcLevel& L, int slot, int k, int b0, int
     int pr = prof_jacobi(false);
     CK(launch_jacobi<T>(order, g, B, cur, bp, oth, nullptr, 0, cf, act, L.shapeT[k], st));
     double cb, cd, cfl;
-    jacobi_cost<T>(order, false, cur == bp, &cb, &cd, &cfl);
+    jacobi_cost<T>(order, g.N, false, cur == bp, &cb, &cd, &cfl);
     if (pr >= 0) h3d_prof_end(c, pr, cb * pts, cd * pts, cfl * pts);
     c->bytes += cb * pts;
     advance();
@@ -570,7 +572,7 @@ static int vcycle_level(heat3d_ctx* c, SdcLevel& L, int slot, int k, int b0, int
     else CK(launch_jacobi<T>(order, g, B, cur, bp, oth, nullptr, 0, cf, act, L.shapeT[k], st));
     if (pr >= 0) {
       double cb, cd, cfl;
-      jacobi_cost<T>(order, upd, false, &cb, &cd, &cfl);
+      jacobi_cost<T>(order, g.N, upd, false, &cb, &cd, &cfl);
       h3d_prof_end(c, pr, cb * pts, cd * pts, cfl * pts);
     }
     if (upd) {
@@ -773,8 +775,11 @@ static int mg_solve_T(heat3d_ctx* c, int lev, int slot, int b0, int B, double* u
     int pr = lev == 0 ? h3d_prof_begin(c, HEAT3D_PROF_RESID64_FINE) : -1;
     CK(launch_resid64<T>(order, g, B, u, us, rhs, bs, c64, bp, cf, L.norms + b0, act, L.shape64, st));
     if (pr >= 0) {
-      // neighbour sums + 2 FMAs (+ the FP64 b' multiply when T is double)
-      double dp = (order == 2 ? 7.0 : order == 4 ? 13.0 : 19.0) + (sizeof(T) == 8 ? 1.0 : 0.0);
+      // neighbour sums + 2 FMAs (large grids: a difference and one or two
+      // FMAs) + the FP64 b' multiply when T is double
+      double dp = (g.N >= fix_min_n(order) ? (order == kCompact ? 3.0 : 2.0)
+                                           : order == 2 ? 7.0 : order == 4 ? 13.0 : 19.0) +
+                  (sizeof(T) == 8 ? 1.0 : 0.0);
       double fl = (order == 2 ? 9.0 : order == 4 ? 16.0 : 22.0) + 1.0;
       h3d_prof_end(c, pr, (16.0 + sizeof(T)) * pts, dp * pts, fl * pts);
     }
@@ -1401,14 +1406,14 @@ static bool tune_log() {
 // percent of the best on a class of grids are left out of it (the deep rings
 // below 127, the one-point tiles' long chunks, kinds 11, 13, 14, 17, 21, 26):
 // a context that is set up beside busy streams pays for every launch here.
-static std::vector<Shape> shape_candidates(int N, bool vec4) {
+static std::vector<Shape> shape_candidates(int order, int N, bool vec4) {
   std::vector<Shape> v;
   auto add = [&](std::initializer_list<int> kinds, std::initializer_list<int> chunks) {
     for (int kind : kinds)
       for (int zc : chunks)
         if (zc <= N) v.push_back(Shape{kind, zc});
   };
-  if (!vec4 && N >= kFixMinN) {  // one kernel, which divides the planes itself
+  if (!vec4 && N >= fix_min_n(order)) {  // one kernel, which divides the planes itself
     v.push_back(Shape{kFixKind, 0});
     return v;
   }
@@ -1437,7 +1442,7 @@ static int autotune_T(heat3d_ctx* c, ShapeTimer& timer) {
       T* b = mgbuf<T>(L, k, 0, 0);
       T* e = mgbuf<T>(L, k, 1, 0);
       T* t = mgbuf<T>(L, k, 2, 0);
-      const std::vector<Shape> cand = shape_candidates(g.N, sizeof(T) == 4);
+      const std::vector<Shape> cand = shape_candidates(L.L.order, g.N, sizeof(T) == 4);
       L.shapeT[k] = cand[0];
       if (cand.size() < 2) continue;
       CK(timer.run((int)cand.size(), c->st, ms, [&](int q) {
@@ -1450,7 +1455,7 @@ static int autotune_T(heat3d_ctx* c, ShapeTimer& timer) {
       L.shapeT[k] = cand[std::min_element(ms.begin(), ms.end()) - ms.begin()];
     }
     const long long fs = L.g.fs;
-    const std::vector<Shape> cand = shape_candidates(L.g.N, false);
+    const std::vector<Shape> cand = shape_candidates(L.L.order, L.g.N, false);
     L.shape64 = cand[0];
     if (cand.size() > 1) {
       CK(timer.run((int)cand.size(), c->st, ms, [&](int q) {

@@ -25,6 +25,10 @@ inline dim3 point_grid(const Grid& g, int B) {
   return dim3((g.N + 31) / 32, (g.N + 7) / 8, g.N * B);
 }
 
+// Planes per thread of the quadrature kernels: as many as leave several
+// blocks for every SM.
+inline int points_per_thread(int N) { return N >= 255 ? 8 : N >= 127 ? 4 : 1; }
+
 // Quadrature integrals of one sweep and (optionally) the collocation residual
 // of the current iterate.  I == nullptr: residual only.
 //
@@ -36,7 +40,12 @@ inline dim3 point_grid(const Grid& g, int B) {
 // each multiplied with 59-bit copies of the matrices (ItemSDC::fI, fQ) as two
 // centred 31-bit digits, and each sum becomes a double once.  Points whose exponents the format does not take go through FP64
 // (plain).  A thread takes a run of kz points along z, which shares the loads
-// of the digits and phi_x phi_y.
+// of the digits and phi_x phi_y; the rows of the two matrices are a loop,
+// which keeps a thread at 64 registers (224 and twice the time without).
+// Error of a sum against exact arithmetic: 0.6-0.8 of the FP64 sums' (rms,
+// M = 3 and 5).  Measured, residual only: 1.25 -> 0.64 ms at 255^3 with M = 5,
+// 0.17 -> 0.10 ms at 127^3, 0.56 -> 0.38 ms at 255^3 with M = 3; the smallest
+// grids take a launch either way.
 struct FixTerm {
   int h, l;
 };
@@ -56,6 +65,39 @@ struct FixSum {
     lo += __mulhi(f.l, c.y);
   }
   __device__ long long value() const { return (hi << 6) + ((mid + 2 * lo) >> 25); }  // of 2^56
+};
+
+// The F values of a point (node stride fs) and its forcing field in digits at
+// their largest exponent E; an even number of terms.
+template <int M>
+struct FixPoint {
+  static constexpr int C = (M + 2) / 2 * 2;
+  FixTerm f[C];
+  int E;
+  __device__ void load(const double* Fb, long long fs, double psi) {
+    double x[C];
+    unsigned key = 0u;
+#pragma unroll
+    for (int q = 0; q < C; ++q) {
+      x[q] = q < M ? Fb[q * fs] : q == M ? psi : 0.0;
+      key = max(key, (unsigned)__double2hiint(x[q]) & 0x7fffffffu);
+    }
+    E = fix_exponent(key);
+#pragma unroll
+    for (int q = 0; q < C; ++q) f[q] = q <= M ? fix_digits(x[q], E) : FixTerm{0, 0};
+  }
+  __device__ bool fits() const { return E <= kFixHi && (E >= kFixLo || E == kFixZero); }
+  // the sum of row c (shared memory, 16-byte aligned) as a double
+  __device__ double row(const int2* c, int fe) const {
+    FixSum s;
+#pragma unroll
+    for (int q = 0; q < C; q += 2) {
+      const int4 v = *reinterpret_cast<const int4*>(c + q);
+      s.add(f[q], make_int2(v.x, v.y));
+      if (q + 1 <= M) s.add(f[q + 1], make_int2(v.z, v.w));
+    }
+    return fix_scale(fix_double(s.value()), E - 1084 + fe);
+  }
 };
 
 // The FP64 form of one point (also the reading of the sums: J_m, I_m, r_m).
@@ -93,7 +135,7 @@ __global__ void __launch_bounds__(256, 4) k_integrals(Grid g, const double* __re
                                                       const double* __restrict__ phi1d,
                                                       unsigned long long* res_bits, const int* active,
                                                       int kz) {
-  constexpr int C = (M + 2) / 2 * 2;  // columns, an even number
+  constexpr int C = FixPoint<M>::C;
   __shared__ __align__(16) int2 cI[M - 1][C], cQ[M - 1][C];
   const int nkz = (g.N + kz - 1) / kz;
   const int b = blockIdx.z / nkz;
@@ -124,36 +166,14 @@ __global__ void __launch_bounds__(256, 4) k_integrals(Grid g, const double* __re
       const double* tb = TAU ? tauS + (long long)b * (M - 1) * fs + idx : nullptr;
       double* Ib = I ? I + (long long)b * (M - 1) * fs + idx : nullptr;
       const double phi = phixy * phi1d[k];
-      FixTerm f[C];
-      int E;
-      {
-        double x[C];
-        unsigned key = 0u;
-#pragma unroll
-        for (int q = 0; q < C; ++q) {
-          x[q] = q < M ? Fb[q * fs] : q == M && forced ? fix_scale(phi, fp) : 0.0;
-          key = max(key, (unsigned)__double2hiint(x[q]) & 0x7fffffffu);
-        }
-        E = fix_exponent(key);
-#pragma unroll
-        for (int q = 0; q < C; ++q) f[q] = q <= M ? fix_digits(x[q], E) : FixTerm{0, 0};
-      }
-      if (!fok || E > kFixHi || (E < kFixLo && E != kFixZero)) {
+      FixPoint<M> p;
+      p.load(Fb, fs, forced ? fix_scale(phi, fp) : 0.0);
+      if (!fok || !p.fits()) {
         const unsigned long long bits = integrals_plain<M>(it, Ub, Fb, tb, Ib, fs, phi, RES);
         mx = bits > mx ? bits : mx;
         continue;
       }
-      const int ke = E - 1084 + fe;
-      auto row = [&](const int2* c) {  // one row's sum as a double
-        FixSum s;
-#pragma unroll
-        for (int q = 0; q < C; q += 2) {
-          const int4 v = *reinterpret_cast<const int4*>(c + q);
-          s.add(f[q], make_int2(v.x, v.y));
-          if (q + 1 <= M) s.add(f[q + 1], make_int2(v.z, v.w));
-        }
-        return fix_scale(fix_double(s.value()), ke);
-      };
+      auto row = [&](const int2* c) { return p.row(c, fe); };
       const double u0 = Ub[0];
       double ctau = 0.0;
       // row m; the one that adds U_0 stands apart (an FP64 addition under a
@@ -239,27 +259,51 @@ __global__ void k_fas_inject(Grid gf, Grid gg, int same, const double* __restric
 // R (one field per item) and into X (the W-solve's start value, item stride
 // xs); max |r| per item into res_bits.
 template <int MF>
-__global__ void k_fas_wresid(Grid gf, int jm, const double* __restrict__ WU,
-                             const double* __restrict__ FF, const ItemSDC* __restrict__ itF,
-                             const double* __restrict__ phif1d, double* __restrict__ R,
-                             double* __restrict__ X, long long xs, unsigned long long* res_bits) {
+__global__ void __launch_bounds__(256, 4) k_fas_wresid(Grid gf, int jm, const double* __restrict__ WU,
+                                                       const double* __restrict__ FF,
+                                                       const ItemSDC* __restrict__ itF,
+                                                       const double* __restrict__ phif1d,
+                                                       double* __restrict__ R, double* __restrict__ X,
+                                                       long long xs, unsigned long long* res_bits, int kz) {
+  constexpr int C = FixPoint<MF>::C;
+  __shared__ __align__(16) int2 cQ[C];  // row jm of dt Q in digits, as k_integrals
+  const int nkz = (gf.N + kz - 1) / kz;
+  const int b = blockIdx.z / nkz;
+  const ItemSDC& it = itF[b];
+  const int tid = threadIdx.y * 32 + threadIdx.x;
+  if (tid < C) cQ[tid] = tid <= MF ? it.fQ[jm - 1][tid] : make_int2(0, 0);
+  const int fe = it.fe, fp = it.fp;
+  const bool fok = it.fok != 0, forced = it.forced != 0;
+  __syncthreads();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  const int b = blockIdx.z / gf.N;
-  const int k = blockIdx.z - b * gf.N;
+  const int k0 = (blockIdx.z - b * nkz) * kz, k1 = min(gf.N, k0 + kz);
   unsigned long long mx = 0ull;
   if (i < gf.N && j < gf.N) {
-    const long long idx = (long long)k * gf.plane + (long long)j * gf.px + i;
-    const double* Wb = WU + (long long)b * MF * gf.fs + idx;
-    const double* Fb = FF + (long long)b * MF * gf.fs + idx;
-    const ItemSDC& it = itF[b];
-    double q = it.gQ[jm] * (phif1d[i] * phif1d[j] * phif1d[k]);
-#pragma unroll
-    for (int p = 0; p < MF; ++p) q = fma(it.dtQ[jm][p], Fb[p * gf.fs], q);
-    const double r = (Wb[0] + q) - Wb[jm * gf.fs];
-    R[(long long)b * gf.fs + idx] = r;
-    X[(long long)b * xs + idx] = r;
-    mx = abs_bits(r);
+    const double phixy = phif1d[i] * phif1d[j];
+#pragma unroll 1
+    for (int k = k0; k < k1; ++k) {
+      const long long idx = (long long)k * gf.plane + (long long)j * gf.px + i;
+      const double* Wb = WU + (long long)b * MF * gf.fs + idx;
+      const double* Fb = FF + (long long)b * MF * gf.fs + idx;
+      const double phi = phixy * phif1d[k];
+      const double w0 = Wb[0], wj = Wb[jm * gf.fs];
+      FixPoint<MF> p;
+      p.load(Fb, gf.fs, forced ? fix_scale(phi, fp) : 0.0);
+      double q;
+      if (fok && p.fits()) {
+        q = p.row(cQ, fe);
+      } else {
+        q = it.gQ[jm] * phi;
+#pragma unroll 1
+        for (int t = 0; t < MF; ++t) q = fma(it.dtQ[jm][t], Fb[t * gf.fs], q);
+      }
+      const double r = (w0 + q) - wj;
+      R[(long long)b * gf.fs + idx] = r;
+      X[(long long)b * xs + idx] = r;
+      const unsigned long long bits = abs_bits(r);
+      mx = bits > mx ? bits : mx;
+    }
   }
   warp_max_to(mx, res_bits + b);
 }
@@ -322,8 +366,7 @@ cudaError_t launch_integrals(int M, const Grid& g, int B, const double* U, const
                              const double* phi1d, unsigned long long* res_bits,
                              const int* active, cudaStream_t st) {
   if (B <= 0) return cudaSuccess;
-  // points per thread: as many as leave several blocks for every SM
-  const int kz = g.N >= 255 ? 8 : g.N >= 127 ? 4 : 1;
+  const int kz = points_per_thread(g.N);
   const dim3 grd((g.N + 31) / 32, (g.N + 7) / 8, (g.N + kz - 1) / kz * B), blk(32, 8);
   switch (M) {
     case 2: start_integrals<2>(grd, blk, st, g, U, F, tauS, I, items, phi1d, res_bits, active, kz); break;
@@ -364,12 +407,13 @@ cudaError_t launch_fas_wresid(int MF, const Grid& gf, int B, int jm, const doubl
                               double* R, double* X, long long xs, unsigned long long* res_bits,
                               cudaStream_t st) {
   if (B <= 0) return cudaSuccess;
-  dim3 grd = point_grid(gf, B), blk(32, 8);
+  const int kz = points_per_thread(gf.N);
+  const dim3 grd((gf.N + 31) / 32, (gf.N + 7) / 8, (gf.N + kz - 1) / kz * B), blk(32, 8);
   switch (MF) {
-    case 2: k_fas_wresid<2><<<grd, blk, 0, st>>>(gf, jm, WU, FF, itF, phif1d, R, X, xs, res_bits); break;
-    case 3: k_fas_wresid<3><<<grd, blk, 0, st>>>(gf, jm, WU, FF, itF, phif1d, R, X, xs, res_bits); break;
-    case 4: k_fas_wresid<4><<<grd, blk, 0, st>>>(gf, jm, WU, FF, itF, phif1d, R, X, xs, res_bits); break;
-    case 5: k_fas_wresid<5><<<grd, blk, 0, st>>>(gf, jm, WU, FF, itF, phif1d, R, X, xs, res_bits); break;
+    case 2: k_fas_wresid<2><<<grd, blk, 0, st>>>(gf, jm, WU, FF, itF, phif1d, R, X, xs, res_bits, kz); break;
+    case 3: k_fas_wresid<3><<<grd, blk, 0, st>>>(gf, jm, WU, FF, itF, phif1d, R, X, xs, res_bits, kz); break;
+    case 4: k_fas_wresid<4><<<grd, blk, 0, st>>>(gf, jm, WU, FF, itF, phif1d, R, X, xs, res_bits, kz); break;
+    case 5: k_fas_wresid<5><<<grd, blk, 0, st>>>(gf, jm, WU, FF, itF, phif1d, R, X, xs, res_bits, kz); break;
     default: return cudaErrorInvalidValue;
   }
   count_launch();

@@ -35,9 +35,12 @@
 // 594 -> 180 us compact, 219 -> 125 us 7-point; refinement residual (wide)
 // 488 -> 208 us; memory time 59 us.  What is left is issue slots: 170 warp
 // instructions per 32 points (wide), 58 % of the slots used, FP64 pipe 42 %,
-// ALU 49 %.  The line at N = 127 (kFixMinN): 62 -> 35 us there (wide; 7-point
-// 33 -> 28); at 63^3 both kernels take a launch's latency and a tile's
-// prologue would cost more than the sums.
+// ALU 49 %.  The line (fix_min_n) lies at 127 for the 7-point and the wide
+// stencil: 33 -> 28 and 62 -> 35 us there; at 63 both kernels take a launch's
+// latency, and the persistent solve repeats the FP64 sums bit for bit.  The
+// compact stencil has no persistent solve and 19 operations: from 63 on (a
+// sweep of four items at 127^3 39.3 -> 36.4 ms by its 63^3 level; one item
+// alone takes the same time either way).
 #pragma once
 #include "fix.cuh"
 
@@ -425,7 +428,7 @@ cudaError_t launch_fix(const Grid& g, int B, int spare, const int* active, unsig
       (long long)((g.N + kFixTX - 1) / kFixTX) * ((g.N + kFixTY - 1) / kFixTY) * g.N * B;
   const long long one = std::max(1, slots.load() - spare);
   const long long waves = B > 1 ? std::max<long long>(1, std::min<long long>(4, total / (one * 24))) : 1;
-  const int run = (int)std::max<long long>(4, (total + waves * one - 1) / (waves * one));
+  const int run = (int)std::max<long long>(2, (total + waves * one - 1) / (waves * one));
   kern<<<(unsigned)((total + run - 1) / run), dim3(32, kFixW), smem, st>>>(g, B, run, active, norm_bits, op);
   return cudaSuccess;
 }

@@ -19,7 +19,7 @@
 //    with each thread's own points of the planes k-R .. k+R in a register
 //    queue; planes by cp.async or TMA (mbarrier per ring slot), k_zq4p as a
 //    producer/consumer pipeline without block barriers.
-//  * k_fix (stencil_fix.cuh; every FP64 stencil of grids with N >= 127): the
+//  * k_fix (stencil_fix.cuh; every FP64 stencil of large grids, fix_min_n): the
 //    neighbour sums in 64-bit fixed point.
 //  * k_zmarch (small grids): one (x, y) column per thread, z-neighbours in a
 //    register queue, x/y neighbours through L1.
@@ -1672,7 +1672,7 @@ cudaError_t run_stencil(const Grid& g, int B, const int* active, unsigned long l
   if (B <= 0 || g.N <= 0) return cudaSuccess;
   int kind = sh.kind;
   if constexpr (sizeof(typename Op::T) == 8) {
-    if (g.N >= kFixMinN) {
+    if (g.N >= fix_min_n(ORDER)) {
       cudaError_t e = launch_fix<ORDER, NORM>(g, B, kind == kFixKind ? sh.zc : 0, active, norm_bits, op, st);
       if (e != cudaSuccess) return e;
       count_launch();
