@@ -10,10 +10,18 @@ constexpr int kFixZero = 64;  // exponent of a set of zeros
 constexpr int kFixLo = 500, kFixHi = 1500;
 
 // Exponent of a set of values (a tile plane, the nodes of a point) from the
-// largest high word (sign cleared) in it.
+// largest high word (sign cleared) in it, the unit of fix_value.
 __host__ __device__ __forceinline__ int fix_exponent(unsigned key) {
   const int e = (int)(key >> 20);
   return e > kFixZero ? e : kFixZero;
+}
+
+// As fix_exponent for a key in which 0 stands for a set of nothing but zeros:
+// a set with any other value, subnormal ones included, lies above kFixZero
+// (and below kFixLo when it is that small).
+__host__ __device__ __forceinline__ int fix_set_exponent(unsigned key) {
+  const int e = fix_exponent(key);
+  return key != 0u && e == kFixZero ? kFixZero + 1 : e;
 }
 
 // The double with high word hi and low word lo in a set of exponent E.

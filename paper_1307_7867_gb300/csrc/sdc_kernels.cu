@@ -82,7 +82,11 @@ struct FixPoint {
       x[q] = q < M ? Fb[q * fs] : q == M ? psi : 0.0;
       key = max(key, (unsigned)__double2hiint(x[q]) & 0x7fffffffu);
     }
-    E = fix_exponent(key);
+    if (key == 0u) {  // zeros, or subnormal values whose high words are 0
+#pragma unroll
+      for (int q = 0; q < C; ++q) key |= __double2loint(x[q]) != 0;
+    }
+    E = fix_set_exponent(key);
 #pragma unroll
     for (int q = 0; q < C; ++q) f[q] = q <= M ? fix_digits(x[q], E) : FixTerm{0, 0};
   }

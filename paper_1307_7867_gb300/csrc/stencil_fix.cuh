@@ -28,8 +28,8 @@
 //   compact: |S2 - 12 c| <= 24 2^(53 + G), G = 5.
 // Planes whose E lies outside [kFixLo, kFixHi] (Inf, NaN, values beyond 1e143
 // or below 1e-157) and coefficients outside 2^+-200 take the FP64 operations
-// of the other kernels, point by point; a plane of zeros (and of values below
-// 2^-1042) counts as zero.
+// of the other kernels, point by point; a plane of nothing but zeros counts as
+// zero.
 //
 // Measured at 255^3 (one item, L2 flushed): damped Jacobi 420 -> 150 us wide,
 // 594 -> 180 us compact, 219 -> 125 us 7-point; refinement residual (wide)
@@ -191,11 +191,18 @@ __global__ void __launch_bounds__(32 * kFixW, 2) k_fix(Grid g, int B, int run, c
     auto key_of = [](double2 v) {
       return max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
     };
-    // largest exponent of plane p (at ring offset s) into keys
+    auto low_of = [](double2 v) { return (unsigned)(__double2loint(v.x) | __double2loint(v.y)); };
+    // largest exponent of plane p (at ring offset s) into keys; 0 is kept for
+    // zeros, subnormal values whose high words are 0 count as 1
     auto scan = [&](int p, int s) {
       unsigned m = key_of(*reinterpret_cast<const double2*>(own + s));
       if (halo_at >= 0) m = max(m, key_of(*reinterpret_cast<const double2*>(ring + halo_at + s)));
       m = __reduce_max_sync(0xffffffffu, m);
+      if (m == 0u) {
+        unsigned l = low_of(*reinterpret_cast<const double2*>(own + s));
+        if (halo_at >= 0) l |= low_of(*reinterpret_cast<const double2*>(ring + halo_at + s));
+        m = __any_sync(0xffffffffu, l != 0u) ? 1u : 0u;
+      }
       if (lane == 0) atomicMax(&keys[p & 7], m);
     };
     // plane p (at ring offset s) into fixed point
@@ -206,7 +213,7 @@ __global__ void __launch_bounds__(32 * kFixW, 2) k_fix(Grid g, int B, int run, c
                          fix_value<G>(__double2hiint(v.y), __double2loint(v.y), E));
     };
     auto decode = [&](int p, int s) {
-      const int E = fix_exponent(keys[p & 7]);
+      const int E = fix_set_exponent(keys[p & 7]);
       fix2(own + s, E);
       if (halo_at >= 0) fix2(ring + halo_at + s, E);
     };
@@ -243,7 +250,7 @@ __global__ void __launch_bounds__(32 * kFixW, 2) k_fix(Grid g, int B, int run, c
       for (int q = 0; q < QL; ++q) {
         int p = k - R + q;
         if (R == 2) p = p == -2 ? 0 : p == N + 1 ? N - 1 : p;
-        e[q] = p < 0 || p >= N ? kFixZero : fix_exponent(keys[p & 7]);
+        e[q] = p < 0 || p >= N ? kFixZero : fix_set_exponent(keys[p & 7]);
         em = max(em, e[q]);
       }
       FixCtl& c = ctl[k & 1];
