@@ -17,30 +17,34 @@
 // significand s becomes s 2^G >> (E - e), truncated towards zero; its unit is
 // 2^(E - 1075 - G).  A point takes the largest E of the planes its stencil
 // touches and shifts each plane's partial sum to it.  All of this depends on
-// the values and their coordinates only, never on the launch.  Errors are
-// relative to the largest value of the tile planes involved: against
-// quad precision at 127^3 the operator is off by 1e-16 of its norm (FP64
-// sums: 1e-14 on sums of sine modes, 1e-16 on random values); values 2^-40
-// and less of their tile plane's largest keep fewer digits of their own than
-// in FP64.  G guard bits
+// the values and their coordinates only, never on the launch.  A value keeps
+// all its 53 bits down to 2^-G of the largest one; a pair of points is summed
+// in integers only if each point's stencil holds such a value (the pair's own
+// two and the neighbours in y are looked at).  Its sums are then off by a few
+// units of 2^-52 of a value that it reads, as FP64 sums are; against quad
+// precision at 127^3 the operator is off by 1e-16 of its norm (FP64 sums:
+// 1e-14 on sums of sine modes, 1e-16 on random values).  The other pairs
+// (0.3-0.5 % of a sum of sine modes, 1 % with the compact stencil: near the
+// boundary and where the field changes sign; two thirds of a narrow hot spot)
+// are redone in FP64 from the field.  G guard bits
 // keep the sums below 2^63:
 //   7-point and wide: |s1 - 6 c| <= 12 2^(53 + G), G = 6;
 //   compact: |S2 - 12 c| <= 24 2^(53 + G), G = 5.
-// Planes whose E lies outside [kFixLo, kFixHi] (Inf, NaN, values beyond 1e143
-// or below 1e-157) and coefficients outside 2^+-200 take the FP64 operations
-// of the other kernels, point by point; a plane of nothing but zeros counts as
-// zero.
+// On planes whose E lies outside [kFixLo, kFixHi] (Inf, NaN, values beyond
+// 1e143 or below 1e-157), or with coefficients outside 2^+-200, every pair is
+// redone; a plane of nothing but zeros counts as zero.
 //
-// Measured at 255^3 (one item, L2 flushed): damped Jacobi 420 -> 150 us wide,
-// 594 -> 180 us compact, 219 -> 125 us 7-point; refinement residual (wide)
-// 488 -> 208 us; memory time 59 us.  What is left is issue slots: 170 warp
-// instructions per 32 points (wide), 58 % of the slots used, FP64 pipe 42 %,
-// ALU 49 %.  The line (fix_min_n) lies at 127 for the 7-point and the wide
-// stencil: 33 -> 28 and 62 -> 35 us there; at 63 both kernels take a launch's
+// Measured at 255^3 (one item; FP64 tiles before, random values and sums of
+// sine modes now): damped Jacobi 423 -> 161 and 167 us wide, 595 -> 197 and
+// 222 us compact, 219 -> 135 and 138 us 7-point; refinement residual (wide)
+// 487 -> 199 and 203 us; memory time 59 us.  A hot spot of width 0.1 takes
+// 465 us (wide), the FP64 redo being two thirds of it.  What is left is issue
+// slots.  The line (fix_min_n) lies at 127 for the 7-point and the wide
+// stencil: 34 -> 29 and 62 -> 38 us there; at 63 both kernels take a launch's
 // latency, and the persistent solve repeats the FP64 sums bit for bit.  The
 // compact stencil has no persistent solve and 19 operations: from 63 on (a
-// sweep of four items at 127^3 39.3 -> 36.4 ms by its 63^3 level; one item
-// alone takes the same time either way).
+// sweep of four items at 127^3 41.0 -> 39.1 ms by its 63^3 level, against
+// 1.19 -> 1.23 ms for five V-cycles on one 63^3 item alone).
 #pragma once
 #include "fix.cuh"
 
@@ -69,6 +73,8 @@ template <int ORDER>
 __host__ __device__ constexpr int fix_plane_size() {
   return (kFixTY + 2 * fix_radius<ORDER>()) * (kFixTX + 4);
 }
+constexpr int kFixBatch = 16;  // pairs that a warp redoes in FP64 at once, a point a lane
+constexpr int kFixSpan = 60;   // planes between two such turns, a multiple of 2R + 1
 template <int ORDER>
 constexpr int fix_smem() {
   return fix_ring<ORDER>() * fix_plane_size<ORDER>() * 8;
@@ -77,9 +83,8 @@ constexpr int fix_smem() {
 struct FixCtl {
   double k1, k2;  // the operator's coefficients, scaled
   int same;       // the planes k - R .. k + R share one exponent (or are zero)
-  int plain;      // the plane is left to FP64
+  int add, sh;    // a value v keeps its 53 bits: (v's high word + add) >> sh
   int shift[5];   // alignment of plane k + d, at d + R
-  int pad;
 };
 
 // A block of 16 warps owns a tile and marches along z, a warp one row and a
@@ -113,8 +118,9 @@ __global__ void __launch_bounds__(32 * kFixW, 2) k_fix(Grid g, int B, int run, c
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double* ring = reinterpret_cast<double*>(smem_raw);  // [NB][SY][SX], doubles or fixed point
   __shared__ unsigned keys[8];   // largest high word of plane p, slot p mod 8
-  __shared__ unsigned todo[32];  // planes left to FP64, a bit each
   __shared__ __align__(16) FixCtl ctl[2];
+  __shared__ unsigned lost[kFixSpan][W];              // pairs left to FP64: a word per plane and row
+  __shared__ unsigned short list[W][kFixBatch + 32];  // plane << 9 | row << 5 | pair, a warp's own
   const int N = g.N, plane = (int)g.plane;
   const int lane = threadIdx.x, warp = threadIdx.y, tid = warp * 32 + lane;
   const int ntx = (N + kFixTX - 1) / kFixTX, nty = (N + TY - 1) / TY;
@@ -261,17 +267,21 @@ __global__ void __launch_bounds__(32 * kFixW, 2) k_fix(Grid g, int B, int run, c
         c.shift[q] = min(em - e[q], 63);
       }
       const bool plain = !coefs || em > kFixHi || (em > kFixZero && em < kFixLo);
+      const bool zero = em == kFixZero && !plain;  // sums and results 0
       c.same = same;
-      c.plain = plain;
-      // exponent of the sums' unit (planes of zeros have sums 0)
-      o.fix_scales(em == kFixZero || plain ? 0 : em - 1075 - G, c.k1, c.k2);
-      if (plain) todo[(k - z0) >> 5] |= 1u << ((k - z0) & 31);
+      // the line is 2^52 in the unit of em; on plain planes no value reaches
+      // it, on planes of zeros every one counts as if
+      const int lim = plain ? 30 : min(20 + em - e[R], 30);
+      c.add = zero ? (int)0x80000000u : 1 << lim;
+      c.sh = zero ? 31 : lim + 1;
+      // exponent of the sums' unit
+      o.fix_scales(zero || plain ? 0 : em - 1075 - G, c.k1, c.k2);
     };
 
     // ---- prologue: planes z0 - R .. z0 - R + NB - 2 under way, those up to
     // z0 + R in fixed point.  Plane p lies in slot (p - z0 + R) mod NB. ----
     if (tid < 8) keys[tid] = 0u;
-    if (tid >= 32 && tid < 64) todo[tid - 32] = 0u;
+    for (int q = tid; q < kFixSpan * W; q += NT) lost[0][q] = 0u;
 #pragma unroll 1
     for (int q = 0; q < NB - 1; ++q) issue(z0 - R + q, q * PS);
     cp_async_wait<NB - 1 - (QL + 1)>();
@@ -299,113 +309,149 @@ __global__ void __launch_bounds__(32 * kFixW, 2) k_fix(Grid g, int B, int run, c
     int base[H];  // ring offsets of the slots QL h .. of the current turn
 #pragma unroll
     for (int h = 0; h < H; ++h) base[h] = h * QL * PS;
-    for (int kb = z0; kb < z1; kb += QL) {
+#pragma unroll 1
+    for (int kc = z0; kc < z1; kc += kFixSpan) {
+      const int ke = min(z1, kc + kFixSpan);
+#pragma unroll 1
+      for (int kb = kc; kb < ke; kb += QL) {
 #pragma unroll
-      for (int uu = 0; uu < QL; ++uu) {
-        const int k = kb + uu;
-        if (k >= z1) break;  // uniform
-        // ring offset of plane k + d
-        auto off = [&](int d) { return base[((uu + d + R + NB) / QL) % H] + ((uu + d + R + NB) % QL) * PS; };
-        typename Op::Ex2 ex;
-        typename Op::Late late;
-        double2 c0;
-        if (live) {
-          ex = o.load2(idx);
-          late = o.late2(idx);
-          if (Op::kFixCentre) c0 = *reinterpret_cast<const double2*>(u + idx);
-        }
-        cp_async_wait<D - 1>();  // plane k + R + 2 has arrived
-        __syncthreads();
-        issue(k - R - 1 + NB, off(-R - 1));
-        if (tid == NT - 32) keys[(k + R + 3) & 7] = 0u;
-        if (k + R + 2 <= zlast) scan(k + R + 2, off(R + 2));
-        if (k + R + 1 <= zlast) decode(k + R + 1, off(R + 1));
-        else if (k + 1 < z1) ghost_plane(k + R + 1, off(R + 1), off(R - 1));
-        if (ghosts && k + 1 < z1) ghost_cells(off(1));
-        if (live) {
-          const FixCtl& cc = ctl[k & 1];
-          auto at = [&](int d, int dy, int dx) {  // pair dx points to the right in row j + dy of plane k + d
-            return *reinterpret_cast<const longlong2*>(own + off(d) + dy * SX + dx);
-          };
-          auto one = [&](int d, int dy, int dx) {
-            return *reinterpret_cast<const long long*>(own + off(d) + dy * SX + dx);
-          };
-          longlong2 d1, d2 = make_longlong2(0, 0);
-          // the sums; al(a, b, d) aligns the partial sums of plane k + d
-          auto sums = [&](auto al) {
-            const longlong2 cr = at(0, 0, 0);
-            const longlong2 c = al(cr.x, cr.y, 0);
-            const long long c60 = 6 * c.x, c61 = 6 * c.y;
-            // n - 6 c and the pairs of the planes k -+ d
-            auto add_z = [&](const longlong2& n, const longlong2& m, const longlong2& p, int d) {
-              const longlong2 v = al(m.x, m.y, -d), w = al(p.x, p.y, d);
-              return make_longlong2(n.x - c60 + (v.x + w.x), n.y - c61 + (v.y + w.y));
-            };
-            const longlong2 ym = at(0, -1, 0), yp = at(0, 1, 0);
-            if constexpr (!CP) {
-              const longlong2 l = at(0, 0, -2), h = at(0, 0, 2);
-              d1 = add_z(al(l.y + cr.y + ym.x + yp.x, cr.x + h.x + ym.y + yp.y, 0), at(-1, 0, 0), at(1, 0, 0), 1);
-              if constexpr (R == 2) {
-                const longlong2 ym2 = at(0, -2, 0), yp2 = at(0, 2, 0);
-                const longlong2 t = add_z(al(l.x + h.x + ym2.x + yp2.x, l.y + h.y + ym2.y + yp2.y, 0),
-                                          at(-2, 0, 0), at(2, 0, 0), 2);
-                d1.x -= t.x >> 4;
-                d1.y -= t.y >> 4;
-              }
-            } else {
-              const longlong2 zm = at(-1, 0, 0), zp = at(1, 0, 0);
-              d1 = add_z(al(one(0, 0, -1) + cr.y + ym.x + yp.x, cr.x + one(0, 0, 2) + ym.y + yp.y, 0), zm, zp, 1);
-              // edges: four of plane k, four of each plane next to it
-              const longlong2 e0 = al((one(0, -1, -1) + ym.y) + (one(0, 1, -1) + yp.y),
-                                      (ym.x + one(0, -1, 2)) + (yp.x + one(0, 1, 2)), 0);
-              auto cross = [&](const longlong2& z, int d) {
-                const longlong2 a = at(d, -1, 0), q = at(d, 1, 0);
-                return al((one(d, 0, -1) + z.y) + (a.x + q.x), (z.x + one(d, 0, 2)) + (a.y + q.y), d);
-              };
-              const longlong2 em1 = cross(zm, -1), ep1 = cross(zp, 1);
-              d2.x = e0.x + em1.x + ep1.x - 2 * c60;
-              d2.y = e0.y + em1.y + ep1.y - 2 * c61;
-            }
-          };
-          if (cc.same) {
-            sums([](long long a, long long q, int) { return make_longlong2(a, q); });
-          } else {
-            sums([&](long long a, long long q, int d) {
-              const int s = cc.shift[d + R];
-              return make_longlong2(a >> s, q >> s);
-            });
+        for (int uu = 0; uu < QL; ++uu) {
+          const int k = kb + uu;
+          if (k >= z1) break;  // uniform
+          // ring offset of plane k + d
+          auto off = [&](int d) { return base[((uu + d + R + NB) / QL) % H] + ((uu + d + R + NB) % QL) * PS; };
+          typename Op::Ex2 ex;
+          typename Op::Late late;
+          double2 c0;
+          if (live) {
+            ex = o.load2(idx);
+            late = o.late2(idx);
+            if (Op::kFixCentre) c0 = *reinterpret_cast<const double2*>(u + idx);
           }
-          const typename Op::Out2 out = o.post2(o.pre2(c0, ex), c0, d1, d2, cc.k1, cc.k2);
-          if (!cc.plain) o.template put2<NORM>(idx, nx, out, late, mx);
+          cp_async_wait<D - 1>();  // plane k + R + 2 has arrived
+          __syncthreads();
+          issue(k - R - 1 + NB, off(-R - 1));
+          if (tid == NT - 32) keys[(k + R + 3) & 7] = 0u;
+          if (k + R + 2 <= zlast) scan(k + R + 2, off(R + 2));
+          if (k + R + 1 <= zlast) decode(k + R + 1, off(R + 1));
+          else if (k + 1 < z1) ghost_plane(k + R + 1, off(R + 1), off(R - 1));
+          if (ghosts && k + 1 < z1) ghost_cells(off(1));
+          if (live) {
+            const FixCtl& cc = ctl[k & 1];
+            auto at = [&](int d, int dy, int dx) {  // pair dx points to the right in row j + dy of plane k + d
+              return *reinterpret_cast<const longlong2*>(own + off(d) + dy * SX + dx);
+            };
+            auto one = [&](int d, int dy, int dx) {
+              return *reinterpret_cast<const long long*>(own + off(d) + dy * SX + dx);
+            };
+            // the pair's own values decide, each of which is in the other's
+            // stencil, or else the neighbours in y of both
+            auto top = [&](int dy, int x) {
+              return (unsigned)reinterpret_cast<const int*>(own + off(0) + dy * SX + x)[1] + (unsigned)cc.add;
+            };
+            bool keep = (top(0, 0) | top(0, 1)) >> cc.sh;
+            if (!keep) {  // seldom
+              keep = (top(-1, 0) | top(1, 0)) >> cc.sh && (top(-1, 1) | top(1, 1)) >> cc.sh;
+              if (!keep) atomicOr(&lost[k - kc][warp], 1u << lane);
+            }
+            longlong2 d1, d2 = make_longlong2(0, 0);
+            // the sums; al(a, b, d) aligns the partial sums of plane k + d
+            auto sums = [&](auto al) {
+              const longlong2 cr = at(0, 0, 0);
+              const longlong2 c = al(cr.x, cr.y, 0);
+              const long long c60 = 6 * c.x, c61 = 6 * c.y;
+              // n - 6 c and the pairs of the planes k -+ d
+              auto add_z = [&](const longlong2& n, const longlong2& m, const longlong2& p, int d) {
+                const longlong2 v = al(m.x, m.y, -d), w = al(p.x, p.y, d);
+                return make_longlong2(n.x - c60 + (v.x + w.x), n.y - c61 + (v.y + w.y));
+              };
+              const longlong2 ym = at(0, -1, 0), yp = at(0, 1, 0);
+              if constexpr (!CP) {
+                const longlong2 l = at(0, 0, -2), h = at(0, 0, 2);
+                d1 = add_z(al(l.y + cr.y + ym.x + yp.x, cr.x + h.x + ym.y + yp.y, 0), at(-1, 0, 0), at(1, 0, 0), 1);
+                if constexpr (R == 2) {
+                  const longlong2 ym2 = at(0, -2, 0), yp2 = at(0, 2, 0);
+                  const longlong2 t = add_z(al(l.x + h.x + ym2.x + yp2.x, l.y + h.y + ym2.y + yp2.y, 0),
+                                            at(-2, 0, 0), at(2, 0, 0), 2);
+                  d1.x -= t.x >> 4;
+                  d1.y -= t.y >> 4;
+                }
+              } else {
+                const longlong2 zm = at(-1, 0, 0), zp = at(1, 0, 0);
+                d1 = add_z(al(one(0, 0, -1) + cr.y + ym.x + yp.x, cr.x + one(0, 0, 2) + ym.y + yp.y, 0), zm, zp, 1);
+                // edges: four of plane k, four of each plane next to it
+                const longlong2 e0 = al((one(0, -1, -1) + ym.y) + (one(0, 1, -1) + yp.y),
+                                        (ym.x + one(0, -1, 2)) + (yp.x + one(0, 1, 2)), 0);
+                auto cross = [&](const longlong2& z, int d) {
+                  const longlong2 a = at(d, -1, 0), q = at(d, 1, 0);
+                  return al((one(d, 0, -1) + z.y) + (a.x + q.x), (z.x + one(d, 0, 2)) + (a.y + q.y), d);
+                };
+                const longlong2 em1 = cross(zm, -1), ep1 = cross(zp, 1);
+                d2.x = e0.x + em1.x + ep1.x - 2 * c60;
+                d2.y = e0.y + em1.y + ep1.y - 2 * c61;
+              }
+            };
+            if (cc.same) {
+              sums([](long long a, long long q, int) { return make_longlong2(a, q); });
+            } else {
+              sums([&](long long a, long long q, int d) {
+                const int s = cc.shift[d + R];
+                return make_longlong2(a >> s, q >> s);
+              });
+            }
+            const typename Op::Out2 out = o.post2(o.pre2(c0, ex), c0, d1, d2, cc.k1, cc.k2);
+            if (keep) o.template put2<NORM>(idx, nx, out, late, mx);
+          }
+          idx += plane;
+          if (tid == NT - 32 && k + 1 < z1) prepare(k + 1);
         }
-        idx += plane;
-        if (tid == NT - 32 && k + 1 < z1) prepare(k + 1);
-      }
-      const int first = base[0];  // the next turn begins QL slots further
+        const int first = base[0];  // the next turn begins QL slots further
 #pragma unroll
-      for (int h = 0; h + 1 < H; ++h) base[h] = base[h + 1];
-      base[H - 1] = first;
+        for (int h = 0; h + 1 < H; ++h) base[h] = base[h + 1];
+        base[H - 1] = first;
+      }
+      // the pairs left to FP64 (no operator writes the field it reads, so their
+      // order is free): a warp takes one row per plane, another one in the next
+      __syncthreads();
+      int n = 0;  // listed
+#pragma unroll 1
+      for (int k0 = kc; k0 < ke; k0 += 32) {
+        const int kl = k0 + lane, row = (warp + kl) & (W - 1);
+        unsigned m = kl < ke ? lost[kl - kc][row] : 0u;
+        if (m) lost[kl - kc][row] = 0u;
+        unsigned todo = __ballot_sync(0xffffffffu, m != 0u);
+#pragma unroll 1
+        for (bool more = true; more;) {
+          const int src = __ffs(todo) - 1;
+          if (todo) {
+            const unsigned w = __shfl_sync(0xffffffffu, m, src);
+            if (w >> lane & 1)
+              list[warp][n + __popc(w & ((1u << lane) - 1))] =
+                  (unsigned short)((k0 + src - kc) << 9 | ((warp + k0 + src) & (W - 1)) << 5 | lane);
+            n += __popc(w);
+            todo &= todo - 1;
+            __syncwarp();
+          }
+          more = todo != 0u;
+#pragma unroll 1
+          while (n >= kFixBatch || (n > 0 && !more && k0 + 32 >= ke)) {
+            const int take = min(n, kFixBatch);
+            n -= take;
+            const int code = list[warp][n + min(lane >> 1, take - 1)];
+            const int x = x0 + 2 * (code & 31) + (lane & 1), y = y0 + (code >> 5 & (W - 1)), z = kc + (code >> 9);
+            if (lane < 2 * take && x < N) {
+              double cc, s1, s2;
+              plain_sums<ORDER>(u, g, x, y, z, cc, s1, s2);
+              const int p = z * plane + y * g.px + x;
+              const double rv = o.apply(p, cc, s1, s2, o.load(p));
+              if (NORM) mx = max(mx, abs_bits(rv));
+            }
+            __syncwarp();
+          }
+        }
+      }
     }
     cp_async_wait<0>();
-    __syncthreads();
-    // planes whose values the fixed-point format does not take, in FP64 (no
-    // operator writes the field it reads, so they can come last)
-#pragma unroll 1
-    for (int c = 0; c <= (z1 - 1 - z0) >> 5; ++c)
-#pragma unroll 1
-      for (unsigned bits = todo[c]; bits; bits &= bits - 1) {
-        const int k = z0 + 32 * c + __ffs(bits) - 1;
-#pragma unroll 1
-        for (int q = 0; q < 2; ++q) {
-          const int x = x0 + lane + 32 * q;
-          if (x >= N || j >= N) continue;
-          double cc, s1, s2;
-          plain_sums<ORDER>(u, g, x, j, k, cc, s1, s2);
-          const int at = k * plane + j * g.px + x;
-          const double rv = o.apply(at, cc, s1, s2, o.load(at));
-          if (NORM) mx = max(mx, abs_bits(rv));
-        }
-      }
     if (NORM) warp_max_to(mx, norm_bits + b);
     __syncthreads();  // the next run's prologue reuses the shared memory
   }

@@ -105,24 +105,41 @@ __device__ __forceinline__ void warp_max_to(unsigned long long v, unsigned long 
 }
 
 // Centre and neighbour sums of one point straight from the field, in the
-// order of every stencil kernel.
+// order of every stencil kernel.  Every load is made (of the point itself or
+// one next to it where the neighbour lies outside), so that all are in flight
+// at once.
 template <int ORDER>
 __device__ __forceinline__ void plain_sums(const double* __restrict__ u, const Grid& g, int i, int j, int k,
                                            double& c, double& s1, double& s2) {
-  c = at(u, g, i, j, k);
-  s1 = ((at(u, g, i - 1, j, k) + at(u, g, i + 1, j, k)) + (at(u, g, i, j - 1, k) + at(u, g, i, j + 1, k))) +
-       (at(u, g, i, j, k - 1) + at(u, g, i, j, k + 1));
+  const int N = g.N, sy = g.px, sz = (int)g.plane;
+  const double* p = u + (long long)k * g.plane + (long long)j * g.px + i;
+  const int x0 = i > 0 ? -1 : 0, x1 = i < N - 1 ? 1 : 0;
+  const int y0 = j > 0 ? -sy : 0, y1 = j < N - 1 ? sy : 0;
+  const int z0 = k > 0 ? -sz : 0, z1 = k < N - 1 ? sz : 0;
+  c = ldg(p);
+  double xm = ldg(p + x0), xp = ldg(p + x1), ym = ldg(p + y0), yp = ldg(p + y1), zm = ldg(p + z0), zp = ldg(p + z1);
   s2 = 0.0;
-  if (ORDER == 4)
-    s2 = ((at(u, g, i - 2, j, k) + at(u, g, i + 2, j, k)) + (at(u, g, i, j - 2, k) + at(u, g, i, j + 2, k))) +
-         (at(u, g, i, j, k - 2) + at(u, g, i, j, k + 2));
-  if (ORDER == kCompact)
-    s2 = (((at(u, g, i - 1, j - 1, k) + at(u, g, i + 1, j - 1, k)) +
-           (at(u, g, i - 1, j + 1, k) + at(u, g, i + 1, j + 1, k))) +
-          ((at(u, g, i - 1, j, k - 1) + at(u, g, i + 1, j, k - 1)) +
-           (at(u, g, i - 1, j, k + 1) + at(u, g, i + 1, j, k + 1)))) +
-         ((at(u, g, i, j - 1, k - 1) + at(u, g, i, j + 1, k - 1)) +
-          (at(u, g, i, j - 1, k + 1) + at(u, g, i, j + 1, k + 1)));
+  if (ORDER == 4) {
+    double xm2 = ldg(p + (i > 1 ? -2 : 0)), xp2 = ldg(p + (i < N - 2 ? 2 : 0));
+    double ym2 = ldg(p + (j > 1 ? -2 * sy : 0)), yp2 = ldg(p + (j < N - 2 ? 2 * sy : 0));
+    double zm2 = ldg(p + (k > 1 ? -2 * sz : 0)), zp2 = ldg(p + (k < N - 2 ? 2 * sz : 0));
+    fix_axis<double, 2>(i, N, c, xm, xp, xm2, xp2);
+    fix_axis<double, 2>(j, N, c, ym, yp, ym2, yp2);
+    fix_axis<double, 2>(k, N, c, zm, zp, zm2, zp2);
+    s2 = ((xm2 + xp2) + (ym2 + yp2)) + (zm2 + zp2);
+  } else {
+    double no = 0.0;
+    fix_axis<double, 1>(i, N, c, xm, xp, no, no);
+    fix_axis<double, 1>(j, N, c, ym, yp, no, no);
+    fix_axis<double, 1>(k, N, c, zm, zp, no, no);
+  }
+  s1 = ((xm + xp) + (ym + yp)) + (zm + zp);
+  if (ORDER == kCompact) {
+    auto edge = [&](int a, int b) { return a != 0 && b != 0 ? ldg(p + a + b) : 0.0; };
+    s2 = (((edge(x0, y0) + edge(x1, y0)) + (edge(x0, y1) + edge(x1, y1))) +
+          ((edge(x0, z0) + edge(x1, z0)) + (edge(x0, z1) + edge(x1, z1)))) +
+         ((edge(y0, z0) + edge(y1, z0)) + (edge(y0, z1) + edge(y1, z1)));
+  }
 }
 
 __device__ __forceinline__ void cp_async16(unsigned s, const void* gmem) {
