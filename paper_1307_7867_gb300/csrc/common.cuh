@@ -11,6 +11,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "fix.cuh"
+
 namespace h3d {
 
 constexpr int kMaxNodes = 5;
@@ -115,7 +117,7 @@ struct ItemSDC {
   double gQ[kMaxNodes];                  // dt * sum_j Q[m][j] g(t0 + dt tau_j)
   double nu;
   // the quadrature kernel's two matrices in fixed point (fix_coefficients),
-  // value = (x 2^31 + y) 2^(fe - 59), |y| <= 2^30: rows of the substep
+  // value = (x 2^31 + y) 2^(fe - kFixBits), |y| <= 2^30: rows of the substep
   // integrals I_m (dtS with -dtm on F_{m+1}) and of the partial sums of J;
   // column M: the forcing, for the field 2^fp Phi, which has the size of the
   // forcing against F (forced = 0: none).  fok = 0: they do not fit the format.
@@ -150,7 +152,7 @@ inline void fix_coefficients(ItemSDC& it, int M) {
   it.fok = s > 1e-60 && s < 1e60 && it.fp > -200 && it.fp < 200;
   it.fe = 0;
   if (!it.fok) return;
-  double scale = 576460752303423488.0;  // 2^59
+  double scale = (double)(1ll << kFixBits);
   while (s >= 1.0) { s *= 0.5; scale *= 0.5; it.fe += 1; }
   while (s < 0.5) { s *= 2.0; scale *= 2.0; it.fe -= 1; }
   auto fixed = [&](double c) { return (long long)(c * scale + (c < 0 ? -0.5 : 0.5)); };

@@ -68,4 +68,30 @@ __device__ __forceinline__ bool fix_coef_ok(double coef) {
   return coef == 0.0 || (e >= 823 && e <= 1223);
 }
 
+// The quadrature's numbers: a value v of kFixBits bits as two centred digits,
+// v = 2^31 h + l, and a sum of products with coefficients (x, y) of two such
+// digits in three parts, 2^62 hi + 2^31 mid + 2^32 lo.  The coefficients'
+// magnitudes add up to 2^kFixBits at most; value() has full scale 2^62.
+constexpr int kFixBits = 59;
+struct FixTerm {
+  int h, l;
+};
+__host__ __device__ __forceinline__ FixTerm fix_digits(long long v) {
+  const int h = (int)((v + (1ll << 30)) >> 31);
+  return FixTerm{h, (int)((unsigned)v - ((unsigned)h << 31))};
+}
+struct FixSum {
+  long long hi = 0, mid = 0;
+  int lo = 0;  // six terms below 2^28
+  __host__ __device__ void add(FixTerm f, int2 c) {
+    hi += (long long)f.h * c.x;
+    mid += (long long)f.h * c.y;
+    mid += (long long)f.l * c.x;
+    lo += (int)(((long long)f.l * c.y) >> 32);
+  }
+  __host__ __device__ long long value() const {
+    return (hi << (124 - 2 * kFixBits)) + ((mid + 2ll * lo) >> (2 * kFixBits - 93));
+  }
+};
+
 }  // namespace h3d

@@ -35,38 +35,17 @@ inline int points_per_thread(int N) { return N >= 255 ? 8 : N >= 127 ? 4 : 1; }
 // With FP64 multiply-adds a point costs 43 FP64 operations (M = 5), 1.40 ms at
 // 255^3 on a pipe of 2 per clock and SM, five times the memory time of its
 // 10 to 14 fields.  The sums run in fixed point instead: the F values of a
-// point (and Phi, scaled by a power of two
-// to the size of the forcing) are brought to the largest exponent among them, 59 bits of
-// each multiplied with 59-bit copies of the matrices (ItemSDC::fI, fQ) as two
-// centred 31-bit digits, and each sum becomes a double once.  Points whose exponents the format does not take go through FP64
-// (plain).  A thread takes a run of kz points along z, which shares the loads
+// point (and Phi, scaled by a power of two to the size of the forcing) are
+// brought to the largest exponent among them, kFixBits bits of each multiplied
+// with copies of the matrices of as many bits (ItemSDC::fI, fQ) as two centred
+// 31-bit digits, and each sum becomes a double once.  Points whose exponents
+// the format does not take go through FP64 (plain).  A thread takes a run of kz points along z, which shares the loads
 // of the digits and phi_x phi_y; the rows of the two matrices are a loop,
 // which keeps a thread at 64 registers (224 and twice the time without).
 // Error of a sum against exact arithmetic: 0.6-0.8 of the FP64 sums' (rms,
 // M = 3 and 5).  Measured, residual only: 1.25 -> 0.64 ms at 255^3 with M = 5,
 // 0.17 -> 0.10 ms at 127^3, 0.56 -> 0.38 ms at 255^3 with M = 3; the smallest
 // grids take a launch either way.
-struct FixTerm {
-  int h, l;
-};
-__device__ __forceinline__ FixTerm fix_digits(double x, int E) {
-  const long long v = fix_value<6>(__double2hiint(x), __double2loint(x), E);
-  const int h = (int)((v + (1ll << 30)) >> 31);
-  return FixTerm{h, (int)(unsigned)v - (int)((unsigned)h << 31)};
-}
-// Sum of products in three parts: 2^62 hi + 2^31 mid + 2^32 lo.
-struct FixSum {
-  long long hi = 0, mid = 0;
-  int lo = 0;
-  __device__ void add(FixTerm f, int2 c) {
-    hi += (long long)f.h * c.x;
-    mid += (long long)f.h * c.y;
-    mid += (long long)f.l * c.x;
-    lo += __mulhi(f.l, c.y);
-  }
-  __device__ long long value() const { return (hi << 6) + ((mid + 2 * lo) >> 25); }  // of 2^56
-};
-
 // The F values of a point (node stride fs) and its forcing field in digits at
 // their largest exponent E; an even number of terms.
 template <int M>
@@ -88,7 +67,9 @@ struct FixPoint {
     }
     E = fix_set_exponent(key);
 #pragma unroll
-    for (int q = 0; q < C; ++q) f[q] = q <= M ? fix_digits(x[q], E) : FixTerm{0, 0};
+    for (int q = 0; q < C; ++q)
+      f[q] = q <= M ? fix_digits(fix_value<kFixBits - 53>(__double2hiint(x[q]), __double2loint(x[q]), E))
+                       : FixTerm{0, 0};
   }
   __device__ bool fits() const { return E <= kFixHi && (E >= kFixLo || E == kFixZero); }
   // the sum of row c (shared memory, 16-byte aligned) as a double
