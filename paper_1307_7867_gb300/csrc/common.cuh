@@ -117,17 +117,24 @@ struct ItemSDC {
   double gQ[kMaxNodes];                  // dt * sum_j Q[m][j] g(t0 + dt tau_j)
   double nu;
   // the quadrature kernel's two matrices in fixed point (fix_coefficients),
-  // value = (x 2^31 + y) 2^(fe - kFixBits), |y| <= 2^30: rows of the substep
-  // integrals I_m (dtS with -dtm on F_{m+1}) and of the partial sums of J;
-  // column M: the forcing, for the field 2^fp Phi, which has the size of the
-  // forcing against F (forced = 0: none).  fok = 0: they do not fit the format.
+  // value = (x 2^31 + y) 2^(fe - kFixBits), |y| <= 2^30, fe that of the row: rows
+  // of the substep integrals I_m (dtS with -dtm on F_{m+1}) and of the partial
+  // sums of J; column M: the forcing, for the field 2^fp Phi, which has the size
+  // of the forcing against F (forced = 0: none).  fok = 0: they do not fit the
+  // format.  weak: the forcing enters some row with a coefficient so small that
+  // F has to be of the size of 2^fp Phi for the format.
   int2 fI[kMaxNodes - 1][kMaxNodes + 1];
   int2 fQ[kMaxNodes - 1][kMaxNodes + 1];
-  int fe, fok, fp, forced;
+  int feI[kMaxNodes - 1], feQ[kMaxNodes - 1];
+  int fok, weak, fp, forced;
 };
 
-// The fixed-point copies: fe is such that the sum of magnitudes of every row
-// of both matrices is below 2^fe.
+// The fixed-point copies.  Numbers are rounded to 2^-kFixBits of their row's
+// sum of magnitudes, F and 2^fp Phi to 2^-60 of the largest of them at a point,
+// so a sum is as accurate as in FP64 if the largest number does not meet a
+// coefficient that is small in its row: Gauss-Lobatto matrices have none below
+// 2^-9 of 2^fe (2^-8.1 at M = 5; others are left to FP64), and for the
+// forcing's, which may be any, there is `weak`.
 inline void fix_coefficients(ItemSDC& it, int M) {
   double gmax = 0.0, smax = 0.0;
   for (int m = 0; m + 1 < M; ++m) {
@@ -136,38 +143,39 @@ inline void fix_coefficients(ItemSDC& it, int M) {
   }
   it.forced = gmax > 0.0;
   it.fp = it.forced ? ilogb(gmax) - ilogb(smax) : 0;
-  auto g = [&](int m) { return ldexp(it.gS[m], -it.fp); };
-  double s = 0.0, cs[kMaxNodes + 1] = {0.0};
-  for (int m = 0; m + 1 < M; ++m) {
-    double ri = it.dtm[m], rq = 0.0;
+  it.fok = it.fp > -200 && it.fp < 200;
+  it.weak = 0;
+  auto coef = [&](int m, int j) { return j < M ? it.dtS[m][j] : ldexp(it.gS[m], -it.fp); };
+  // row m of a matrix: the sums of the rows first .. m of dtS, less dtm on F_{m+1}
+  auto row = [&](int first, int m, bool less, int2* out, int& fe) {
+    double s = 0.0, c[kMaxNodes + 1];
     for (int j = 0; j <= M; ++j) {
-      const double v = j < M ? it.dtS[m][j] : g(m);
-      cs[j] += v;
-      ri += fabs(v);
-      rq += fabs(cs[j]);
+      c[j] = less && j == m + 1 ? -it.dtm[m] : 0.0;
+      for (int q = first; q <= m; ++q) c[j] += coef(q, j);
+      s += fabs(c[j]);
     }
-    s = fmax(s, fmax(ri, rq));
-  }
-  s *= 1.0 + 1e-9;  // over the copies' own rounding
-  it.fok = s > 1e-60 && s < 1e60 && it.fp > -200 && it.fp < 200;
-  it.fe = 0;
-  if (!it.fok) return;
-  double scale = (double)(1ll << kFixBits);
-  while (s >= 1.0) { s *= 0.5; scale *= 0.5; it.fe += 1; }
-  while (s < 0.5) { s *= 2.0; scale *= 2.0; it.fe -= 1; }
-  auto fixed = [&](double c) { return (long long)(c * scale + (c < 0 ? -0.5 : 0.5)); };
-  auto split = [](long long v) {
-    const long long hi = (v + (1ll << 30)) >> 31;
-    return make_int2((int)hi, (int)(v - hi * (1ll << 31)));
+    s *= 1.0 + 1e-9;  // over the roundings
+    fe = 0;
+    if (!(s > 1e-60 && s < 1e60)) {
+      it.fok = 0;
+      return;
+    }
+    fe = ilogb(s) + 1;
+    for (int j = 0; j < M; ++j)
+      if (c[j] != 0.0 && fabs(c[j]) < ldexp(1.0, fe - 9)) it.fok = 0;
+    if (it.forced && fabs(c[M]) < ldexp(1.0, fe - 7)) it.weak = 1;
+    auto fixed = [&](double v) { return llround(ldexp(v, kFixBits - fe)); };
+    for (int j = 0; j <= M; ++j) {
+      long long v = less && j == m + 1 ? -fixed(it.dtm[m]) : 0;
+      for (int q = first; q <= m; ++q) v += fixed(coef(q, j));
+      const long long hi = (v + (1ll << 30)) >> 31;
+      out[j] = make_int2((int)hi, (int)(v - hi * (1ll << 31)));
+    }
   };
-  long long cum[kMaxNodes + 1] = {0};
-  for (int m = 0; m + 1 < M; ++m)
-    for (int j = 0; j <= M; ++j) {
-      const long long v = fixed(j < M ? it.dtS[m][j] : g(m));
-      cum[j] += v;
-      it.fI[m][j] = split(j == m + 1 ? v - fixed(it.dtm[m]) : v);
-      it.fQ[m][j] = split(cum[j]);
-    }
+  for (int m = 0; m + 1 < M; ++m) {
+    row(m, m, true, it.fI[m], it.feI[m]);
+    row(0, m, false, it.fQ[m], it.feQ[m]);
+  }
 }
 
 // FAS transfer data between the fine (F) and coarse (G) levels.

@@ -72,7 +72,7 @@ __device__ __forceinline__ bool fix_coef_ok(double coef) {
 // v = 2^31 h + l, and a sum of products with coefficients (x, y) of two such
 // digits in three parts, 2^62 hi + 2^31 mid + 2^32 lo.  The coefficients'
 // magnitudes add up to 2^kFixBits at most; value() has full scale 2^62.
-constexpr int kFixBits = 59;
+constexpr int kFixBits = 61;
 struct FixTerm {
   int h, l;
 };

@@ -39,13 +39,15 @@ inline int points_per_thread(int N) { return N >= 255 ? 8 : N >= 127 ? 4 : 1; }
 // brought to the largest exponent among them, kFixBits bits of each multiplied
 // with copies of the matrices of as many bits (ItemSDC::fI, fQ) as two centred
 // 31-bit digits, and each sum becomes a double once.  Points whose exponents
-// the format does not take go through FP64 (plain).  A thread takes a run of kz points along z, which shares the loads
+// the format does not take go through FP64 (plain), and where a coefficient of
+// the forcing is tiny (fix_coefficients) those whose F is small against it.  A thread takes a run of kz points along z, which shares the loads
 // of the digits and phi_x phi_y; the rows of the two matrices are a loop,
 // which keeps a thread at 64 registers (224 and twice the time without).
-// Error of a sum against exact arithmetic: 0.6-0.8 of the FP64 sums' (rms,
-// M = 3 and 5).  Measured, residual only: 1.25 -> 0.64 ms at 255^3 with M = 5,
-// 0.17 -> 0.10 ms at 127^3, 0.56 -> 0.38 ms at 255^3 with M = 3; the smallest
-// grids take a launch either way.
+// Error of a sum against exact arithmetic: 0.3-1.0 of the FP64 sums' (rms and
+// largest, M = 2 to 5, node values alike, spread over 2^40, one much larger
+// than the others, all far below the forcing).  Measured, residual only: 1.25
+// -> 0.66 ms at 255^3 with M = 5, 0.17 -> 0.10 ms at 127^3, 0.56 -> 0.40 ms at
+// 255^3 with M = 3; the smallest grids take a launch either way.
 // The F values of a point (node stride fs) and its forcing field in digits at
 // their largest exponent E; an even number of terms.
 template <int M>
@@ -53,19 +55,22 @@ struct FixPoint {
   static constexpr int C = (M + 2) / 2 * 2;
   FixTerm f[C];
   int E;
+  bool low;  // every F is below 1/16 of the largest number
   __device__ void load(const double* Fb, long long fs, double psi) {
     double x[C];
-    unsigned key = 0u;
+    unsigned key = 0u, keyF = 0u;
 #pragma unroll
     for (int q = 0; q < C; ++q) {
       x[q] = q < M ? Fb[q * fs] : q == M ? psi : 0.0;
       key = max(key, (unsigned)__double2hiint(x[q]) & 0x7fffffffu);
+      if (q == M - 1) keyF = key;
     }
     if (key == 0u) {  // zeros, or subnormal values whose high words are 0
 #pragma unroll
       for (int q = 0; q < C; ++q) key |= __double2loint(x[q]) != 0;
     }
     E = fix_set_exponent(key);
+    low = (int)(keyF >> 20) < E - 4;
 #pragma unroll
     for (int q = 0; q < C; ++q)
       f[q] = q <= M ? fix_digits(fix_value<kFixBits - 53>(__double2hiint(x[q]), __double2loint(x[q]), E))
@@ -122,6 +127,7 @@ __global__ void __launch_bounds__(256, 4) k_integrals(Grid g, const double* __re
                                                       int kz) {
   constexpr int C = FixPoint<M>::C;
   __shared__ __align__(16) int2 cI[M - 1][C], cQ[M - 1][C];
+  __shared__ int eI[M - 1], eQ[M - 1];
   const int nkz = (g.N + kz - 1) / kz;
   const int b = blockIdx.z / nkz;
   if (active && !active[b]) return;  // uniform over the block
@@ -131,10 +137,13 @@ __global__ void __launch_bounds__(256, 4) k_integrals(Grid g, const double* __re
     const int m = tid / C, j = tid - m * C;
     cI[m][j] = j <= M ? it.fI[m][j] : make_int2(0, 0);
     cQ[m][j] = j <= M ? it.fQ[m][j] : make_int2(0, 0);
+    if (j == 0) {
+      eI[m] = it.feI[m];
+      eQ[m] = it.feQ[m];
+    }
   }
-  const int fe = it.fe, fp = it.fp;
-  const bool forced = it.forced != 0;
-  const bool fok = it.fok != 0;
+  const int fp = it.fp;
+  const bool forced = it.forced != 0, fok = it.fok != 0, weak = it.weak != 0;
   __syncthreads();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -153,12 +162,11 @@ __global__ void __launch_bounds__(256, 4) k_integrals(Grid g, const double* __re
       const double phi = phixy * phi1d[k];
       FixPoint<M> p;
       p.load(Fb, fs, forced ? fix_scale(phi, fp) : 0.0);
-      if (!fok || !p.fits()) {
+      if (!fok || !p.fits() || (weak && p.low)) {
         const unsigned long long bits = integrals_plain<M>(it, Ub, Fb, tb, Ib, fs, phi, RES);
         mx = bits > mx ? bits : mx;
         continue;
       }
-      auto row = [&](const int2* c) { return p.row(c, fe); };
       const double u0 = Ub[0];
       double ctau = 0.0;
       // row m; the one that adds U_0 stands apart (an FP64 addition under a
@@ -166,13 +174,13 @@ __global__ void __launch_bounds__(256, 4) k_integrals(Grid g, const double* __re
       auto substep = [&](int m, auto first) {
         const double tau = TAU ? tb[m * fs] : 0.0;
         if (I) {
-          double Im = row(cI[m]);
+          double Im = p.row(cI[m], eI[m]);
           if (TAU) Im += tau;
           if (decltype(first)::value) Im += u0;
           Ib[m * fs] = Im;
         }
         if (RES) {
-          double rv = (u0 - Ub[(m + 1) * fs]) + row(cQ[m]);
+          double rv = (u0 - Ub[(m + 1) * fs]) + p.row(cQ[m], eQ[m]);
           if (TAU) rv += ctau += tau;
           const unsigned long long bits = abs_bits(rv);
           mx = bits > mx ? bits : mx;
@@ -257,8 +265,8 @@ __global__ void __launch_bounds__(256, 4) k_fas_wresid(Grid gf, int jm, const do
   const ItemSDC& it = itF[b];
   const int tid = threadIdx.y * 32 + threadIdx.x;
   if (tid < C) cQ[tid] = tid <= MF ? it.fQ[jm - 1][tid] : make_int2(0, 0);
-  const int fe = it.fe, fp = it.fp;
-  const bool fok = it.fok != 0, forced = it.forced != 0;
+  const int fe = it.feQ[jm - 1], fp = it.fp;
+  const bool fok = it.fok != 0, forced = it.forced != 0, weak = it.weak != 0;
   __syncthreads();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -276,7 +284,7 @@ __global__ void __launch_bounds__(256, 4) k_fas_wresid(Grid gf, int jm, const do
       FixPoint<MF> p;
       p.load(Fb, gf.fs, forced ? fix_scale(phi, fp) : 0.0);
       double q;
-      if (fok && p.fits()) {
+      if (fok && p.fits() && !(weak && p.low)) {
         q = p.row(cQ, fe);
       } else {
         q = it.gQ[jm] * phi;
