@@ -8,8 +8,6 @@
 // coarse_fused.cuh), bitwise the same as the launch sequence.
 #include "coarse_fused.cuh"
 
-#include <atomic>
-
 namespace h3d {
 namespace {
 
@@ -30,16 +28,9 @@ constexpr size_t small_smem_max(size_t tsize) {
 
 template <typename T, int ORDER>
 cudaError_t launch_small(const SmallArgs<T>& a, int B, size_t smem, cudaStream_t st) {
-  // the shared-memory opt-in once per process (one device) and for every
-  // depth: the call waits for other streams' kernels, up to a tenth of a
-  // second when they keep the GPU full
-  static std::atomic<bool> set{false};
-  if (!set.load()) {
-    cudaError_t e = cudaFuncSetAttribute(k_vcycle_small<T, ORDER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)small_smem_max(sizeof(T)));
-    if (e != cudaSuccess) return e;
-    set.store(true);
-  }
+  static PerDevice once;  // for every depth
+  const cudaError_t e = opt_in_smem(once, k_vcycle_small<T, ORDER>, (int)small_smem_max(sizeof(T)));
+  if (e != cudaSuccess) return e;
   k_vcycle_small<T, ORDER><<<B, 512, smem, st>>>(a);
   count_launch();
   return cudaGetLastError();

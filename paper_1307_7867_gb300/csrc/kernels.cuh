@@ -4,6 +4,9 @@
 // item 0 of the launch), skips item b when active != nullptr and active[b] == 0,
 // and returns cudaGetLastError() of the launch.
 #pragma once
+#include <atomic>
+#include <mutex>
+
 #include "common.cuh"
 
 namespace h3d {
@@ -27,6 +30,55 @@ struct Shape {
   int kind = 0;
   int zc = 16;
 };
+
+// What a kernel needs before its first launch on a device (shared-memory
+// opt-in, resident blocks): setup(dev, &value) runs once for each device that
+// is current when get() is called, and its value is kept.  Function attributes
+// belong to a device; setting one waits for other streams' kernels, up to a
+// tenth of a second when they keep the GPU full.
+class PerDevice {
+ public:
+  template <typename Setup>
+  cudaError_t get(int* value, Setup&& setup) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kDevices) return setup(dev, value);
+    if (!ready_[dev].load(std::memory_order_acquire)) {
+      std::lock_guard<std::mutex> lk(mu_);
+      if (!ready_[dev].load(std::memory_order_relaxed)) {
+        const cudaError_t rc = setup(dev, &value_[dev]);
+        if (rc != cudaSuccess) return rc;
+        ready_[dev].store(true, std::memory_order_release);
+      }
+    }
+    *value = value_[dev];
+    return cudaSuccess;
+  }
+
+ private:
+  static constexpr int kDevices = 64;
+  std::mutex mu_;
+  std::atomic<bool> ready_[kDevices] = {};
+  int value_[kDevices] = {};
+};
+// Opt-in to `smem` bytes of dynamic shared memory, once per device.
+template <typename Kernel>
+cudaError_t opt_in_smem(PerDevice& once, Kernel kern, int smem) {
+  int unused = 0;
+  return once.get(&unused, [&](int, int*) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  });
+}
+// Blocks of a kernel that fit the whole device at once.
+template <typename Kernel>
+cudaError_t resident_blocks(int dev, Kernel kern, int threads, size_t smem, int* slots) {
+  int sms = 0, per_sm = 0;
+  cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+  *slots = sms * per_sm;
+  return e;
+}
 
 // Process-wide count of kernel launches (every launcher calls it once per launch).
 void count_launch();

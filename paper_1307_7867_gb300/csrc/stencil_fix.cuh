@@ -467,19 +467,16 @@ cudaError_t launch_fix(const Grid& g, int B, int spare, const int* active, unsig
                        const Op& op, cudaStream_t st) {
   constexpr int smem = fix_smem<ORDER>();
   auto kern = k_fix<ORDER, NORM, Op>;
-  static std::atomic<int> slots{0};  // resident blocks on the whole GPU (one device)
-  if (slots.load() == 0) {
-    int dev = 0, sms = 0, bps = 0;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess) e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, 32 * kFixW, smem);
-    if (e != cudaSuccess) return e;
-    slots.store(std::max(1, sms * bps));
-  }
+  static PerDevice once;
+  int slots = 0;
+  const cudaError_t e = once.get(&slots, [&](int dev, int* n) {
+    const cudaError_t rc = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    return rc == cudaSuccess ? resident_blocks(dev, kern, 32 * kFixW, smem, n) : rc;
+  });
+  if (e != cudaSuccess) return e;
   const long long total =
       (long long)((g.N + kFixTX - 1) / kFixTX) * ((g.N + kFixTY - 1) / kFixTY) * g.N * B;
-  const long long one = std::max(1, slots.load() - spare);
+  const long long one = std::max(1, slots - spare);
   const long long waves = B > 1 ? std::max<long long>(1, std::min<long long>(4, total / (one * 24))) : 1;
   const int run = (int)std::max<long long>(2, (total + waves * one - 1) / (waves * one));
   kern<<<(unsigned)((total + run - 1) / run), dim3(32, kFixW), smem, st>>>(g, B, run, active, norm_bits, op);

@@ -39,7 +39,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <atomic>
 #include <type_traits>
 
 #include "kernels.cuh"
@@ -807,20 +806,16 @@ __global__ void __launch_bounds__(32 * TYT) k_tile(Grid g, int nzc, int zc, cons
 }
 
 // One tiled launch: TYT warps per block, RY rows per thread, D planes of
-// prefetch.  Rings above 48 KB need the shared-memory opt-in (set once).
+// prefetch.  Rings above 48 KB need the shared-memory opt-in.
 template <int ORDER, int TYT, int RY, int D, bool NORM, typename Op>
 cudaError_t launch_tile(const Grid& g, int B, int nzc, int zc, const int* active,
                         unsigned long long* norm_bits, const Op& op, cudaStream_t st) {
   using T = typename Op::T;
   constexpr int smem = tile_smem_bytes<T, ORDER, TYT, RY, D>();
   if (smem > 48 * 1024) {
-    static std::atomic<bool> set{false};  // set once per process (one device)
-    if (!set.load()) {
-      cudaError_t e = cudaFuncSetAttribute(k_tile<ORDER, TYT, RY, D, NORM, Op>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      if (e != cudaSuccess) return e;
-      set.store(true);
-    }
+    static PerDevice once;
+    const cudaError_t e = opt_in_smem(once, k_tile<ORDER, TYT, RY, D, NORM, Op>, smem);
+    if (e != cudaSuccess) return e;
   }
   dim3 blk(32, TYT, 1);
   dim3 grd((g.N + 31) / 32, (g.N + TYT * RY - 1) / (TYT * RY), nzc * B);
@@ -1085,13 +1080,9 @@ cudaError_t launch_tile4(const Grid& g, int B, int nzc, int zc, const int* activ
                          cudaStream_t st) {
   constexpr int smem = tile4_smem<ORDER, TYT, RY, D>();
   if (smem > 48 * 1024) {
-    static std::atomic<bool> set{false};  // set once per process (one device)
-    if (!set.load()) {
-      cudaError_t e = cudaFuncSetAttribute(k_tile4<ORDER, TYT, RY, D, Op>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      if (e != cudaSuccess) return e;
-      set.store(true);
-    }
+    static PerDevice once;
+    const cudaError_t e = opt_in_smem(once, k_tile4<ORDER, TYT, RY, D, Op>, smem);
+    if (e != cudaSuccess) return e;
   }
   dim3 blk(32, TYT, 1);
   dim3 grd((g.N + 127) / 128, (g.N + TYT * RY - 1) / (TYT * RY), nzc * B);
@@ -1631,26 +1622,19 @@ cudaError_t launch_zq4(const Grid& g, int B, int zc, const int* active, const Op
   if constexpr (TMA == 2) kern = k_zq4p<ORDER, TYT, DEEP, Op>;
   else kern = k_zq4<ORDER, TYT, DEEP, TMA, Op>;
   if (smem > 48 * 1024) {
-    static std::atomic<bool> set{false};  // set once per process (one device)
-    if (!set.load()) {
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      if (e != cudaSuccess) return e;
-      set.store(true);
-    }
+    static PerDevice once;
+    const cudaError_t e = opt_in_smem(once, kern, smem);
+    if (e != cudaSuccess) return e;
   }
   const int tiles = ((g.N + 127) / 128) * ((g.N + TYT - 1) / TYT) * B;
   if (zc <= 0) {
-    static std::atomic<int> slots{0};  // resident blocks on the whole GPU (one device)
-    if (slots.load() == 0) {
-      int dev = 0, sms = 0, bps = 0;
-      cudaError_t e = cudaGetDevice(&dev);
-      if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, threads, smem);
-      if (e != cudaSuccess) return e;
-      slots.store(std::max(1, sms * bps));
-    }
+    static PerDevice once;
+    int slots = 0;
+    const cudaError_t e =
+        once.get(&slots, [&](int dev, int* n) { return resident_blocks(dev, kern, threads, smem, n); });
+    if (e != cudaSuccess) return e;
     const int waves = zc < 0 ? -zc : 1;
-    const int nfit = std::max(1, waves * slots.load() / tiles);
+    const int nfit = std::max(1, waves * slots / tiles);
     zc = (g.N + nfit - 1) / nfit;
   }
   zc = std::min(zc, g.N);
