@@ -29,7 +29,6 @@
 // launch guarantees that all blocks are resident at once.
 
 #include <algorithm>
-#include <atomic>
 
 #include "../../include/heat3d.h"
 #include "coarse_fused.cuh"
@@ -474,29 +473,43 @@ __global__ void k_barrier_selftest(PersistCtl* ctl, int absent, int* out) {
 template <typename T, int ORDER>
 cudaError_t launch_order(const PersistArgs<T>& A, int nblk, size_t smem, cudaStream_t st) {
   auto kern = k_mg_persist<T, ORDER>;
-  // shared-memory opt-in and resident blocks, once per process (one device)
-  // for the largest shared memory seen: host work of every small solve else
-  static std::atomic<int> slots{0};
-  static std::atomic<size_t> opted{0};
-  if (slots.load() == 0 || opted.load() < smem) {
-    const size_t want = std::max(smem, opted.load());
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)want);
+  // Shared memory grows with the batch.  Above 48 KB (thousands of items) it
+  // needs the opt-in, once per device and for whatever a block can have, so
+  // that no call lowers another's; the resident blocks of the last size on a
+  // device are kept per host thread (a query of every small solve else).
+  cudaError_t err = cudaSuccess;
+  if (smem > 48 * 1024) {
+    static PerDevice once;
+    int unused = 0;
+    err = once.get(&unused, [&](int dev, int*) {
+      int most = 0;
+      cudaFuncAttributes fa;
+      cudaError_t e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+      if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kern);
+      if (e != cudaSuccess) return e;
+      return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  most - (int)fa.sharedSizeBytes);
+    });
     if (err != cudaSuccess) return err;
-    int dev = 0, nsm = 0, per_sm = 0;
-    if ((err = cudaGetDevice(&dev)) != cudaSuccess) return err;
-    if ((err = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-      return err;
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPersistThreads, want);
-    if (err != cudaSuccess) return err;
-    if (per_sm < 1) return cudaErrorCooperativeLaunchTooLarge;
-    slots.store(per_sm * nsm);
-    opted.store(want);
   }
-  nblk = std::max(1, std::min(nblk, slots.load()));
+  struct Last {
+    int dev = -1;
+    size_t smem = 0;
+    int slots = 0;
+  };
+  static thread_local Last last;
+  int dev = 0;
+  if ((err = cudaGetDevice(&dev)) != cudaSuccess) return err;
+  if (last.dev != dev || last.smem != smem) {
+    int slots = 0;
+    if ((err = resident_blocks(dev, kern, kPersistThreads, smem, &slots)) != cudaSuccess) return err;
+    if (slots < 1) return cudaErrorCooperativeLaunchTooLarge;
+    last = Last{dev, smem, slots};
+  }
+  nblk = std::max(1, std::min(nblk, last.slots));
   PersistArgs<T> arg = A;
   void* args[] = {&arg};
-  cudaError_t err = cudaLaunchCooperativeKernel((const void*)kern, dim3(nblk), dim3(kPersistThreads),
-                                                args, smem, st);
+  err = cudaLaunchCooperativeKernel((const void*)kern, dim3(nblk), dim3(kPersistThreads), args, smem, st);
   count_launch();
   return err;
 }
