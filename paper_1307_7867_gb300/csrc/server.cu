@@ -124,7 +124,10 @@ struct heat3d_server {
   // step run alone (guarded by mu, cv_gate): they load kernels, time launch
   // shapes and capture graphs, and the driver makes a first use of a kernel
   // wait until the GPU is idle, which beside busy groups it may not be for a
-  // second.
+  // second.  Three 63^3 requests to a new group while three of 127^3 and one of
+  // 255^3 run: 1.1-1.8 -> 0.9-1.2 s, all of them 1.9 -> 1.3 s.  The others wait
+  // meanwhile; a 127^3 request beside groups of 63^3 and 31^3 that evict each
+  // other all the time takes 0.55 s (0.58 without the gate, 0.43 alone).
   std::condition_variable cv_gate;
   int stepping = 0, setups = 0;  // steps in flight; set-ups waiting or running
   bool setting_up = false;
@@ -223,7 +226,9 @@ static Group* get_group(heat3d_server* s, int N) {
   g->chunk = chunk;
   // A small grid's kernels are a few microseconds each; at an equal priority
   // each would wait for a large grid's blocks, which fill the GPU for up to a
-  // whole kernel.  The smaller the grid, the higher its stream's priority.
+  // whole kernel.  The smaller the grid, the higher its stream's priority
+  // (three 63^3 requests beside three of 127^3 and one of 255^3, groups set up:
+  // 0.41-0.49 -> 0.31 s, 127^3 1.30 -> 1.22 s, 255^3 0.86 -> 0.94 s).
   int lo = 0, hi = 0;
   cudaDeviceGetStreamPriorityRange(&lo, &hi);
   const int prio = std::max(hi, lo - (N <= 63 ? 2 : N <= 127 ? 1 : 0));
@@ -238,12 +243,14 @@ static Group* get_group(heat3d_server* s, int N) {
     s->pool.release(chunk);
     return nullptr;
   }
-  // its large FP64 kernels leave some of the GPU to the other groups' (the
-  // blocks of 12 SMs of 152)
+  // its large FP64 kernels leave a twelfth of the GPU to the other groups', two
+  // blocks per SM (127^3 above 1.25 -> 1.22 s, 63^3 0.32 -> 0.31 s)
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->cfg.device);
   SdcLevel& L = g->ctx->lv[0];
-  if (L.shape64.kind == kFixKind) L.shape64.zc = 24;
+  if (L.shape64.kind == kFixKind) L.shape64.zc = 2 * (sms / 12);
   for (int k = 0; k < L.nmg; ++k)
-    if (L.shapeT[k].kind == kFixKind) L.shapeT[k].zc = 24;
+    if (L.shapeT[k].kind == kFixKind) L.shapeT[k].zc = 2 * (sms / 12);
   char* p = chunk + (ws + 255) / 256 * 256;
   Grid gr = make_grid(N);
   g->ucur = (double*)p;
@@ -398,9 +405,13 @@ static void group_loop(heat3d_server* s, Group* g) {
       if (s->stop) return;
       if (g->stop && g->incoming.empty() && g->active() == 0) return;
       // An idle group starts with the request that woke it and takes what has
-      // arrived by then in its next round, so that the same submissions make
-      // the same batches (the FP32 cycles per refinement step are chosen for a
-      // batch) however fast this thread wakes.
+      // arrived by then in its next round.  The FP32 cycles per refinement step
+      // are chosen for a batch, so in mixed precision a result depends on its
+      // batch within the solver's tolerance.  Taking all that has arrived made
+      // the first batch depend on how fast this thread wakes: twelve requests at
+      // once gave 3 to 5 different results in 25 passes, with errors 4.3e-11 to
+      // 5.0e-11, against one result now, in the same time (196 ms; a step of one
+      // request more).  Later batches still depend on what arrives during a step.
       if (g->active() == 0) {
         inc.push_back(g->incoming.front());
         g->incoming.pop_front();
