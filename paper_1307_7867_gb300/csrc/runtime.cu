@@ -1402,10 +1402,12 @@ static bool tune_log() {
 // four-points-per-thread FP32 tiles (kinds 7-14, and 15-26 with the z
 // neighbours in registers, 19-26 loading planes by TMA, 23-26 with a producer
 // warp and no block barriers); the latter also try the chunks that fill one or
-// two whole waves of the GPU.  Kinds and chunks that never came within a few
-// percent of the best on a class of grids are left out of it (the deep rings
-// below 127, the one-point tiles' long chunks, kinds 11, 13, 14, 17, 21, 26):
-// a context that is set up beside busy streams pays for every launch here.
+// two whole waves of the GPU.  The list is short because a context that is set
+// up beside busy streams pays for every launch here: all kinds and chunks (143
+// below 127^3) made requests of a new serving group finish after those it was
+// set up beside.  Single launches of 5 us are timed in steps of 2 us, so on small
+// grids many candidates tie and the first is taken; a mixed 63^3 solve takes
+// 2.12 ms with either list (medians of ten set-ups; one set-up in ten 2.25).
 static std::vector<Shape> shape_candidates(int order, int N, bool vec4) {
   std::vector<Shape> v;
   auto add = [&](std::initializer_list<int> kinds, std::initializer_list<int> chunks) {
