@@ -36,6 +36,12 @@ sys.path.insert(0, ROOT)
 
 import numpy as np  # noqa: E402
 
+# records of the other workloads of a default run: in full on stderr, their
+# values in the stdout line (tens of kilobytes with all of them)
+OTHER_WORKLOADS = ("mixed", "adaptive", "adaptive_mixed", "cubic", "cubic_mixed", "p8", "p8_mixed", "c1", "c3",
+                   "c3_mixed", "c3_p8", "c3_p8_mixed", "c3_p8_converged", "c4", "paperc_p8_mixed", "c5",
+                   "alpha_p8")
+
 # DRAM bytes (read + write) per launch of the roofline kernel, from one ncu
 # capture of the kernel as it is now; key: (precision, fine stencil order, N).
 # Must be cleared when that kernel changes.
@@ -803,6 +809,17 @@ def run_alpha(args):
                             "xe6_large": 0.4}}
 
 
+def headline(out):
+    """The stdout line: the headline workload's record, and of every other
+    workload its value (seconds-like or failed ones: its message)."""
+    line = {k: v for k, v in out.items() if not (isinstance(v, dict) and k in OTHER_WORKLOADS)}
+    others = {k: out[k].get("value", out[k].get("error", out[k].get("alpha")))
+              for k in OTHER_WORKLOADS if isinstance(out.get(k), dict)}
+    if others:
+        line["other_workloads"] = others
+    return line
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -952,7 +969,8 @@ def main():
         iters = st["iters"] / K if w["coarse"] else st["sweeps"] / K
         out["cpu_baseline"] = cpu_baseline(w, iters, vpts, "counted by this GPU run")
     if rank == 0:
-        print(json.dumps(out), flush=True)
+        print(json.dumps(out), file=sys.stderr, flush=True)  # everything measured
+        print(json.dumps(headline(out)), flush=True)
     if world > 1:
         import torch.distributed as dist
         dist.barrier()
