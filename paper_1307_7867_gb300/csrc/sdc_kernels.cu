@@ -29,25 +29,6 @@ inline dim3 point_grid(const Grid& g, int B) {
 // blocks for every SM.
 inline int points_per_thread(int N) { return N >= 255 ? 8 : N >= 127 ? 4 : 1; }
 
-// Quadrature integrals of one sweep and (optionally) the collocation residual
-// of the current iterate.  I == nullptr: residual only.
-//
-// With FP64 multiply-adds a point costs 43 FP64 operations (M = 5), 1.40 ms at
-// 255^3 on a pipe of 2 per clock and SM, five times the memory time of its
-// 10 to 14 fields.  The sums run in fixed point instead: the F values of a
-// point (and Phi, scaled by a power of two to the size of the forcing) are
-// brought to the largest exponent among them, kFixBits bits of each multiplied
-// with copies of the matrices of as many bits (ItemSDC::fI, fQ) as two centred
-// 31-bit digits, and each sum becomes a double once.  Points whose exponents
-// the format does not take go through FP64 (plain), and where a coefficient of
-// the forcing is tiny (fix_coefficients) those whose F is small against it.  A thread takes a run of kz points along z, which shares the loads
-// of the digits and phi_x phi_y; the rows of the two matrices are a loop,
-// which keeps a thread at 64 registers (224 and twice the time without).
-// Error of a sum against exact arithmetic: 0.3-1.0 of the FP64 sums' (rms and
-// largest, M = 2 to 5, node values alike, spread over 2^40, one much larger
-// than the others, all far below the forcing).  Measured, residual only: 1.25
-// -> 0.66 ms at 255^3 with M = 5, 0.17 -> 0.10 ms at 127^3, 0.56 -> 0.40 ms at
-// 255^3 with M = 3; the smallest grids take a launch either way.
 // The F values of a point (node stride fs) and its forcing field in digits at
 // their largest exponent E; an even number of terms.
 template <int M>
@@ -116,6 +97,26 @@ __device__ __noinline__ unsigned long long integrals_plain(const ItemSDC& it, co
   return mx;
 }
 
+// Quadrature integrals of one sweep and (optionally) the collocation residual
+// of the current iterate.  I == nullptr: residual only.
+//
+// With FP64 multiply-adds a point costs 43 FP64 operations (M = 5), 1.40 ms at
+// 255^3 on a pipe of 2 per clock and SM, five times the memory time of its 10
+// to 14 fields.  The sums run in fixed point instead: the F values of a point
+// (and Phi, scaled by a power of two to the size of the forcing) are brought to
+// the largest exponent among them, kFixBits bits of each multiplied with copies
+// of the matrices of as many bits (ItemSDC::fI, fQ) as two centred 31-bit
+// digits, and each sum becomes a double once.  Points whose exponents the
+// format does not take go through FP64 (plain), and where a coefficient of the
+// forcing is tiny (fix_coefficients) those whose F is small against it.  A
+// thread takes a run of kz points along z, which shares the loads of the digits
+// and phi_x phi_y; the rows of the two matrices are a loop, which keeps a
+// thread at 64 registers (224 and twice the time without).  Error of a sum
+// against exact arithmetic: 0.3-1.0 of the FP64 sums' (rms and largest, M = 2
+// to 5, node values alike, spread over 2^40, one much larger than the others,
+// all far below the forcing).  Measured, residual only: 1.25 -> 0.66 ms at
+// 255^3 with M = 5, 0.17 -> 0.10 ms at 127^3, 0.56 -> 0.40 ms at 255^3 with M =
+// 3; the smallest grids take a launch either way.
 template <int M, bool TAU, bool RES>
 __global__ void __launch_bounds__(256, 4) k_integrals(Grid g, const double* __restrict__ U,
                                                       const double* __restrict__ F,

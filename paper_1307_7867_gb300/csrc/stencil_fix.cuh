@@ -39,12 +39,14 @@
 // 222 us compact, 219 -> 135 and 138 us 7-point; refinement residual (wide)
 // 487 -> 199 and 203 us; memory time 59 us.  A hot spot of width 0.1 takes
 // 465 us (wide), the FP64 redo being two thirds of it.  What is left is issue
-// slots.  The line (fix_min_n) lies at 127 for the 7-point and the wide
-// stencil: 34 -> 29 and 62 -> 38 us there; at 63 both kernels take a launch's
-// latency, and the persistent solve repeats the FP64 sums bit for bit.  The
-// compact stencil has no persistent solve and 19 operations: from 63 on (a
-// sweep of four items at 127^3 41.0 -> 39.1 ms by its 63^3 level, against
-// 1.19 -> 1.23 ms for five V-cycles on one 63^3 item alone).
+// slots: 192 warp instructions per 32 points (wide; 237 compact, 169
+// 7-point), 54-59 % of the slots used, ALU 45-53 %, FP64 pipe 39-47 %.  The
+// line (fix_min_n) lies at 127 for the 7-point and the wide stencil: 34 -> 29
+// and 62 -> 38 us there; at 63 both kernels take a launch's latency, and the
+// persistent solve repeats the FP64 sums bit for bit.  The compact stencil
+// has no persistent solve and 19 operations: from 63 on (a sweep of four
+// items at 127^3 41.0 -> 39.1 ms by its 63^3 level, against 1.19 -> 1.23 ms
+// for five V-cycles on one 63^3 item alone).
 #pragma once
 #include "fix.cuh"
 
