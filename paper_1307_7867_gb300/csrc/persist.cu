@@ -473,12 +473,13 @@ __global__ void k_barrier_selftest(PersistCtl* ctl, int absent, int* out) {
 template <typename T, int ORDER>
 cudaError_t launch_order(const PersistArgs<T>& A, int nblk, size_t smem, cudaStream_t st) {
   auto kern = k_mg_persist<T, ORDER>;
-  // Shared memory grows with the batch.  Above 48 KB (thousands of items) it
-  // needs the opt-in, once per device and for whatever a block can have, so
-  // that no call lowers another's; the resident blocks of the last size on a
-  // device are kept per host thread (a query of every small solve else).
+  // Shared memory grows with the batch.  With thousands of items it needs the
+  // opt-in (above 48 KB, the kernel's static part included), once per device
+  // and for whatever a block can have, so that no call lowers another's; the
+  // resident blocks of the last size on a device are kept per host thread (a
+  // query of every small solve else).
   cudaError_t err = cudaSuccess;
-  if (smem > 48 * 1024) {
+  if (smem > 32 * 1024) {
     static PerDevice once;
     int unused = 0;
     err = once.get(&unused, [&](int dev, int*) {

@@ -48,7 +48,8 @@ static cudaError_t fake_memset(void*, int, size_t, cudaStream_t) { return cudaSu
 static cudaError_t fake_launch(const void* k, dim3, dim3, void**, size_t smem, cudaStream_t) {
   std::lock_guard<std::mutex> lk(mu);
   const auto it = allowed.find(k);
-  return smem <= (size_t)(it == allowed.end() ? 48 * 1024 : it->second) ? cudaSuccess : cudaErrorInvalidValue;
+  // without an opt-in, 48 KB for static and dynamic shared memory together
+  return smem <= (size_t)(it == allowed.end() ? 48 * 1024 - 64 : it->second) ? cudaSuccess : cudaErrorInvalidValue;
 }
 #define cudaFuncSetAttribute fake_set
 #define cudaFuncGetAttributes fake_fattr
@@ -101,7 +102,7 @@ def test_batches_of_different_size(tmp_path):
     exe = str(tmp_path / "p")
     subprocess.run([nvcc, "-gencode", "arch=compute_103a,code=sm_103a", "-std=c++17", "-Xptxas", "-O0", f"-I{ROOT}",
                     f"-I{ROOT}/include", "-o", exe, str(tmp_path / "p.cu")], check=True, capture_output=True)
-    for small in (4, 12000):
+    for small in (4, 10060, 12000):  # 9 KB, 8 bytes below 48 KB, 56 KB
         for hold_at in range(8):
             out = subprocess.run([exe, str(hold_at), str(small)], capture_output=True, text=True, check=True).stdout
             assert out.strip() == "0", (small, hold_at)
